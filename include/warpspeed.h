@@ -12,9 +12,10 @@
  * Table designs (§2.2, §5): double hashing over 8-slot buckets (DoubleHT) and
  * power-of-two-choice over 32-slot buckets (P2HT), each optionally with a
  * 16-bit fingerprint per slot (the "(M)" metadata variants, §4.3).  Same-key
- * writers serialise on one lock bit of the key's primary bucket, held in an
- * external array (§4.1, §5 "Concurrency and metadata"); queries take no lock
- * and read each slot with one 128-bit load (§4.2).
+ * writers serialise on one lock bit, chosen by the key's hash from an external
+ * array (§4.1, §5 "Concurrency and metadata"; the paper has one bit per
+ * bucket); queries take no lock and read each slot with one 128-bit load
+ * (§4.2).
  *
  * Conventions shared by every entry point
  * ---------------------------------------

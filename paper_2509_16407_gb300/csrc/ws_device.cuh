@@ -52,7 +52,7 @@ struct Counters {
 struct TableView {
   Slot* slots;    // nb * B slots
   u16* tags;      // nb * B tags (metadata tables) or null
-  u32* locks;     // one bit per bucket
+  u32* locks;     // 2^(64 - lock_shift) lock bits (see TileOps::lock_of)
   Counters* ctr;
   u64 nb_mask;    // nb - 1
   u64 nb_front;   // iceberg: front-yard buckets [0, nb_front), backyard [nb_front, nb)
@@ -60,6 +60,7 @@ struct TableView {
   u64 seed1, seed2;
   u32 pmax;       // double hashing: buckets a probe sequence may visit (<= nb)
   u32 spin_limit; // lock attempts before giving up
+  u32 lock_shift; // lock bit of a key: h2 >> lock_shift
   int shortcut;   // P2: no erase ever ran, so the primary-fill shortcut is exact
   int preload;    // the lane path with cp.async snapshots (1), or every op to the tiles (0)
   int phased;     // bulk-synchronous mode: weak cacheable probe loads, no locks (see WS_OPT_PHASED)
@@ -135,8 +136,8 @@ __device__ __forceinline__ void ld_tags16_weak(const u16* p, u64& a, u64& b) {
 
 // 128-bit compare-and-swap of a whole slot (relaxed: the pair itself is the
 // published datum; a lock release or a release store orders it where needed).
-// Returns true on success.
-__device__ __forceinline__ bool cas_slot(Slot* p, u64 ek, u64 ev, u64 nk, u64 nv) {
+// Returns true on success; *seen gets the key found there.
+__device__ __forceinline__ bool cas_slot(Slot* p, u64 ek, u64 ev, u64 nk, u64 nv, u64* seen = nullptr) {
   u64 ok, ov;
   asm volatile(
       "{\n\t.reg .b128 d, c, s;\n\t"
@@ -147,6 +148,7 @@ __device__ __forceinline__ bool cas_slot(Slot* p, u64 ek, u64 ev, u64 nk, u64 nv
       : "=l"(ok), "=l"(ov)
       : "l"(ek), "l"(ev), "l"(nk), "l"(nv), "l"(p)
       : "memory");
+  if (seen) *seen = ok;
   return ok == ek && ov == ev;
 }
 

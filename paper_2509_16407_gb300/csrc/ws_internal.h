@@ -62,7 +62,7 @@ struct DeviceGuard {
 
 struct ws_table {
   ws::TableView tv;
-  wsi::u64 nb = 0, B = 0, S = 0;
+  wsi::u64 nb = 0, B = 0, S = 0, lock_words = 0;
   int T = 0, scheme = 0, meta = 0, device = 0, num_sms = 0;
   uint32_t pmax = 0, spin = 0;
   int never_erased = 1;

@@ -37,10 +37,9 @@
 //     (stability, §2.1: keys never move);
 //   * plain insert / upsert calls on double-hashing tables need no lock at all
 //     (no erase runs in the same call, see do_upsert);
-//   * otherwise an absent key is inserted under the lock bit of its primary
-//     bucket b_0 (one bit per bucket in an external array; iceberg: the front
-//     bucket): insert-if-unique ops take it before probing, add / max /
-//     replace only once the key is proven absent.  The holder re-reads and
+//   * otherwise an absent key is inserted under its lock bit (chosen by the
+//     key's hash, see lock_of): insert-if-unique ops take it before probing,
+//     add / max / replace only once the key is proven absent.  The holder re-reads and
 //     claims a free slot with one 128-bit CAS that publishes key and value
 //     together (metadata tables: a 16-bit CAS on the tag, then a 128-bit
 //     store of the pair).  The lock makes same-key inserters agree on one location (the
@@ -705,8 +704,16 @@ struct TileOps {
       ptx::st_u64_relaxed(vp, V);
   }
 
-  // One test-and-test-and-set attempt on the lock bit of bucket b by the
-  // leader lane; the outcome is returned on every lane of the tile.
+  // Lock bit of a key.  A lock serialises inserters of one key, which share
+  // its bit; inserters of different keys agree through the claim CAS, so the
+  // bits need not follow the buckets (see ws_table_create_ex for their
+  // number).  With one bit per bucket a table that L2 holds had about one op
+  // in flight per bit (155k lanes on the 131k buckets of 2^22 slots), and most
+  // of an insert's time went into missed locks.
+  __device__ static __forceinline__ u64 lock_of(const TableView& tv, u64 h2) { return h2 >> tv.lock_shift; }
+
+  // One test-and-test-and-set attempt on lock bit b by the leader lane; the
+  // outcome is returned on every lane of the tile.
   __device__ static __forceinline__ bool try_lock(const TableView& tv, const TileCtx<T>& c, u64 b) {
     int ok = 0;
     if (c.tl == 0) {
@@ -764,6 +771,47 @@ struct TileOps {
     if (ch == 0 && !free0) ch = 1;
     else if (ch == 1 && !free1) ch = 0;
     return (ch == 0 ? free0 : free1) ? ch : -1;
+  }
+
+  // A lane's claim of free slot idx (observed tag fk, or pair {fk, fv}) for
+  // (K, V).  When another op takes an EMPTY slot first, the bucket's next slot
+  // is the next candidate: EMPTY slots are a suffix of the bucket and the lost
+  // CAS has shown idx taken, so the lane goes on from there, below slot
+  // `limit`, instead of probing the sequence again.  Inserters of one bucket
+  // arrive together on tables that are small against the launch: when 45,875
+  // keys build a 2^16-slot DoubleHT, 5 are in flight per bucket, and the build
+  // took 60 us with a new probe after each lost claim, 22 us with this.  (With
+  // more lock bits and lane passes, 6.7M inserts into a 2^23-slot IcebergHT(M)
+  // went from 1387 to 650 us, 209,715 into a 2^22-slot P2HT(M) from 145 to
+  // 62 us.)  holder: only this lane may insert K (it holds K's lock).  Returns
+  // 1 claimed, 2 the slot at idx holds K (plain tables), 0 lost.
+  __device__ static __forceinline__ int lane_claim(const TableView& tv, u64& idx, u64 limit, u64 fk, u64 fv, u64 K,
+                                                   u64 V, bool holder) {
+    for (;;) {
+      if (META) {
+        const u16 got = ptx::cas_tag(tv.tags + idx, (u16)fk, key_tag(K));
+        if (got == (u16)fk) {
+          ptx::st_slot_relaxed(tv.slots + idx, K, V);
+          return 1;
+        }
+        if (got == key_tag(K) && !holder) return 0;  // perhaps K itself, its pair not written yet
+        if (fk != TAG_EMPTY) return 0;
+      } else {
+        u64 got;
+        if (ptx::cas_slot(tv.slots + idx, fk, fv, K, V, &got)) return 1;
+        if (got == K) return 2;
+        if (fk != KEY_EMPTY) return 0;
+        fv = 0;  // EMPTY slots hold {0, 0}
+      }
+      if (++idx >= limit) return 0;
+    }
+  }
+  // How far a claim may move on from slot idx: to the end of its bucket, but
+  // under two choices only while the bucket stays below the 3/4 threshold
+  // (beyond it the other bucket may be the less loaded one).
+  __device__ static __forceinline__ u64 claim_limit(u64 idx) {
+    const u64 first = idx & ~(u64)(B - 1);
+    return first + (SCHEME == SCHEME_P2 ? (u64)FILL_SHORTCUT : (u64)B);
   }
 
   // ----------------------------------------------------------------------
@@ -846,10 +894,10 @@ struct TileOps {
     // inserting this very key -- probe again lock-free: once the key is
     // present its slot never moves, so the update needs no lock.  This keeps
     // a batch's many copies of a hot key from queueing on one lock bit.
-    const u64 b0 = bucket(tv, h1, h2, 0);
+    const u64 lk = lock_of(tv, h2);
     // bulk-synchronous mode: distinct keys per call, nothing to serialise
     for (u32 tries = 0, ns = 0; !phased;) {
-      if (try_lock(tv, c, b0)) break;
+      if (try_lock(tv, c, lk)) break;
       const Hit again = find(tv, c, K, h1, h2, no_pre());
       if (again.found) {
         if (c.tl == 0) apply(tv, again.idx, op, V);
@@ -876,7 +924,7 @@ struct TileOps {
         break;
       }
     }
-    if (!phased) unlock(tv, c, b0, st == ST_INSERTED);
+    if (!phased) unlock(tv, c, lk, st == ST_INSERTED);
     return st;
   }
 
@@ -1114,9 +1162,9 @@ struct TileOps {
       st = ST_FULL;
       return 1;
     }
-    const bool ok = ch == 0 ? ptx::cas_slot(tv.slots + ls.ff_idx, ls.ff_k, ls.ff_v, K, V)
-                            : ptx::cas_slot(tv.slots + ls.f1_idx, ls.f1_k, ls.f1_v, K, V);
-    if (!ok) {
+    u64 idx = ch == 0 ? ls.ff_idx : ls.f1_idx;
+    if (lane_claim(tv, idx, claim_limit(idx), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V, true) !=
+        1) {
       fresh = false;
       return -1;
     }
@@ -1242,17 +1290,15 @@ struct TileOps {
         }
       }
     }
-    bool ok;
-    if (META) {
-      const u16 expect = (u16)fk;
-      ok = ptx::cas_tag(tv.tags + fidx, expect, key_tag(K)) == expect;
-      if (ok) ptx::st_slot_relaxed(tv.slots + fidx, K, V);
-    } else {
-      ok = ptx::cas_slot(tv.slots + fidx, fk, fv, K, V);
-    }
-    if (!ok) {
+    const int got = lane_claim(tv, fidx, claim_limit(fidx), fk, fv, K, V, opk == LW_INSERT_LOCKED);
+    if (got == 0) {
       fresh = false;
       return -1;
+    }
+    if (got == 2) {  // another op of the call has just inserted K here
+      apply(tv, fidx, op, V);
+      st = ST_FOUND;
+      return 1;
     }
     ++dcount;
     st = ST_INSERTED;
@@ -1286,6 +1332,7 @@ __device__ __forceinline__ void count_failure(const TableView& tv, u8 st) {
 // -------------------------------------------------------------------------
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
+constexpr int kChunkPasses = 4;  // 32-op chunks: lane passes of an insert whose lock or claim was lost before the tiles
 constexpr int kLaneRestarts = 2;  // streaming lane: restarts of an op after a lost CAS before the tiles
 
 struct WarpSmem {
@@ -1363,36 +1410,38 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   // absent one goes to the tiles, which lock and rescan.  A lane that misses
   // the lock also leaves absent keys to the tiles, which wait for it.
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || kRounds;
-  const u64 b0 = Ops::bucket(tv, h1, h2, 0);
+  const u64 b0 = Ops::bucket(tv, h1, h2, 0), lk = Ops::lock_of(tv, h2);
   bool locked = false;
   if (kLaneLock && lane_ok && !done && opk == Ops::LW_UPDATE_ONLY && (op == OP_INSERT || tv.phased)) {
-    locked = tv.phased || Ops::lane_lock(tv, b0);  // bulk-synchronous: no locks
+    locked = tv.phased || Ops::lane_lock(tv, lk);  // bulk-synchronous: no locks
     if (locked) opk = Ops::LW_INSERT_LOCKED;
   }
   int snap_wave = -1;
 
+  constexpr int kPasses = (KIND == KIND_UPSERT || KIND == KIND_MIXED) ? kChunkPasses : 1;
+  bool again = false;  // run the op through the lane path once more
   if (kRounds) {
     // Whole-bucket rounds: eight buckets per round, one op's bucket per copy
     // instruction (lane s copies slot s), each scanned with two votes.
     // Pass 0 reads b_0 of every open op, pass 1 b_1 of the ops still open;
     // the lane owning an op settles it.  An op that proved its key absent
-    // without holding b_0's lock (its one attempt found the lock taken, or
-    // an add / max / replace that probed lock-free) tries the lock once more
-    // after the rounds and, holding it, reads its buckets again (now in L2)
-    // and claims; only ops that still miss the lock, or lose a CAS, go to
-    // the tiles.
-    for (int attempt = 0; attempt < 2; ++attempt) {
+    // without holding its lock (its attempt found the lock taken, or an add /
+    // max / replace that probed lock-free) tries the lock again after the
+    // rounds and reads its buckets again (now in L2), with the lock or
+    // without it (the holder may be inserting this very key); a holder whose
+    // claim was lost reads again too.  Only ops still open after kPasses
+    // go to the tiles.
+    for (int attempt = 0; attempt < kPasses; ++attempt) {
       bool open = lane_ok && !done;
-      if (attempt == 1) {
-        const bool retry = open && kLaneLock && opk == Ops::LW_UPDATE_ONLY && fresh;
-        const bool got = retry && Ops::lane_lock(tv, b0);
-        if (got) {
-          locked = true;
-          opk = Ops::LW_INSERT_LOCKED;
+      if (attempt > 0) {
+        open = open && kLaneLock && again;
+        if (open && !locked) {
+          locked = Ops::lane_lock(tv, lk);
+          if (locked) opk = Ops::LW_INSERT_LOCKED;
         }
-        open = got;
         if (!__any_sync(0xffffffffu, open)) break;
       }
+      again = false;
       u32 occ0 = 0;
       int f0 = -1;
       u64 f0k = 0, f0v = 0;
@@ -1488,18 +1537,26 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
               st = ST_FULL;
               done = true;
             } else {
-              const u64 idx = ch == 0 ? b0 * 32 + (u64)f0 : bc * 32 + (u64)fs;
-              if (ptx::cas_slot(tv.slots + idx, ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K, V)) {
+              u64 idx = ch == 0 ? b0 * 32 + (u64)f0 : bc * 32 + (u64)fs;
+              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K, V,
+                                  true) == 1) {
                 ++dcount;
                 st = ST_INSERTED;
                 done = true;
+              } else {
+                again = true;
               }
             }
+          } else {
+            again = true;  // absent, and this op holds no lock
           }
         }
       }
-      if (locked && !tv.phased) Ops::lane_unlock(tv, b0, done && st == ST_INSERTED);  // after the claim
-      locked = false;
+      // a holder keeps its lock while it goes round again
+      if (locked && (done || !again || attempt + 1 == kPasses)) {
+        if (!tv.phased) Ops::lane_unlock(tv, lk, done && st == ST_INSERTED);  // after the claim
+        locked = false;
+      }
     }
   }
 
@@ -1519,33 +1576,34 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
                         : (SCHEME == SCHEME_DOUBLE) ? (tv.lane_waves > 0 ? (u32)tv.lane_waves : 4u)
                         : (SCHEME == SCHEME_ICEBERG) ? 3u
                                                      : 2u;
-  // Pass 0 follows every open op.  Pass 1 reads again, under b_0's lock, the
-  // ops whose keys proved absent without it (a lane that missed the lock, or
-  // an add / max / replace that probed lock-free): by then the lock's holder
-  // has usually finished, and the lane settles the op from L2-resident lines
-  // instead of handing it to a tile that would spin on the lock.
-  bool relock = false;
-  for (int pass = 0; pass < 2; ++pass) {
-    if (pass == 1) {
-      bool again = false;
-      if (relock) {
-        again = Ops::lane_lock(tv, b0);
-        if (again) {
-          locked = true;
-          opk = Ops::LW_INSERT_LOCKED;
-          ls.ff_set = false;
-          ls.ff_idx = ls.ff_k = ls.ff_v = 0;
-          ls.occ0 = ls.occ1 = 0;
-          ls.f1_set = false;
-          ls.tsum = 0;
-          ls.f1_idx = ls.f1_k = 0;
+  // Pass 0 follows every open op.  Later passes read again the ops whose keys
+  // proved absent without the lock (a lane that missed the lock, or an add /
+  // max / replace that probed lock-free) -- under the lock if it is free now,
+  // else lock-free, since its holder may be inserting this very key -- and the
+  // holders whose claim was lost, from L2-resident lines, instead of handing
+  // them to tiles that spin on the lock.
+  for (int pass = 0; pass < kPasses; ++pass) {
+    bool run = lane_ok && !done;
+    if (pass > 0) {
+      run = run && again;
+      if (!__any_sync(0xffffffffu, run)) break;
+      if (run) {
+        if (!locked && opk == Ops::LW_UPDATE_ONLY) {
+          locked = Ops::lane_lock(tv, lk);
+          if (locked) opk = Ops::LW_INSERT_LOCKED;
         }
+        fresh = true;
+        ls.ff_set = false;
+        ls.ff_idx = ls.ff_k = ls.ff_v = 0;
+        ls.occ0 = ls.occ1 = 0;
+        ls.f1_set = false;
+        ls.tsum = 0;
+        ls.f1_idx = ls.f1_k = 0;
       }
-      if (!__any_sync(0xffffffffu, again)) break;
-      lane_ok = again;  // the other open ops (a sequence longer than the waves) go to the tiles
     }
+    again = false;
     for (u32 w = 0; w < max_waves; ++w) {
-      const bool want = lane_ok && !done;
+      const bool want = run && !done;
       const unsigned wmask = __ballot_sync(0xffffffffu, want);
       if (!wmask) break;
       sm.bw[lane] = want ? Ops::bucket(tv, h1, h2, w) : 0;
@@ -1578,17 +1636,22 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
             Ops::lane_wave(tv, p, K, V, op, opk, w, sm.bw[lane], ls, out, st, dcount, fresh, KIND != KIND_ERASE);
         if (r > 0) {
           done = true;
-        } else if (r == -2 && kLaneLock && pass == 0 && !locked) {
-          relock = true;  // absent, and this op holds no lock
-          lane_ok = false;
         } else if (r < 0) {
-          lane_ok = false;
+          run = false;
+          if ((r == -2 && kLaneLock && !locked) ||
+              (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE)))
+            again = true;  // absent without the lock, or a lost claim
+          else
+            lane_ok = false;
         }
       }
       __syncwarp();  // the next wave overwrites the snapshots
     }
-    if (locked && !tv.phased) Ops::lane_unlock(tv, b0, done && st == ST_INSERTED);  // after the claim
-    locked = false;
+    // a holder keeps its lock while it goes round again
+    if (locked && (done || !again || pass + 1 == kPasses)) {
+      if (!tv.phased) Ops::lane_unlock(tv, lk, done && st == ST_INSERTED);  // after the claim
+      locked = false;
+    }
   }
   // the tile path may reuse a snapshot only if it is still of b_0 and fresh
   const unsigned pre_mask = __ballot_sync(0xffffffffu, snap_wave == 0 && fresh);
@@ -1777,7 +1840,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
             state = L_PARKED;
           } else {
             if (kLaneLock && opk == Ops::LW_UPDATE_ONLY && (op == OP_INSERT || tv.phased)) {
-              locked = tv.phased || Ops::lane_lock(tv, Ops::bucket(tv, h1, h2, 0));
+              locked = tv.phased || Ops::lane_lock(tv, Ops::lock_of(tv, h2));
               if (locked) opk = Ops::LW_INSERT_LOCKED;
             }
             state = L_ACTIVE;
@@ -1844,7 +1907,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           if (st >= ST_FULL) count_failure(tv, st);
           state = L_EMPTY;
         } else if (r == -2 && kLaneLock && !locked &&
-                   Ops::lane_lock(tv, Ops::bucket(tv, sm.h1[lane], sm.h2[lane], 0))) {
+                   Ops::lane_lock(tv, Ops::lock_of(tv, sm.h2[lane]))) {
           // absent without the lock: now holding b_0's lock, follow the
           // sequence again from b_0 and insert from what it reads
           locked = true;
@@ -1876,7 +1939,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           w = Ops::kLines ? ls.next_w : w + 1;
         }
         if (state != L_ACTIVE && locked) {
-          if (!tv.phased) Ops::lane_unlock(tv, Ops::bucket(tv, sm.h1[lane], sm.h2[lane], 0), wrote);  // after the claim
+          if (!tv.phased) Ops::lane_unlock(tv, Ops::lock_of(tv, sm.h2[lane]), wrote);  // after the claim
           locked = false;
         }
       }

@@ -1,0 +1,57 @@
+"""Inserts whose inserters meet: tables built from nothing by one call, several
+ops in flight per bucket and per lock bit, with and without copies of a key.
+Exactly one copy of a key reports INSERTED, the map equals the oracle's and
+the layout rules hold (EMPTY slots a suffix, no duplicate, two-choice and
+iceberg early exits).  Needs a GPU."""
+import numpy as np
+import pytest
+
+import workloads as W
+from tests._gpu import DESIGNS, DESIGN_IDS, check_layout, dev, host
+
+pytestmark = pytest.mark.gpu
+
+CASES = [(s, m, 0) for s, m in DESIGNS] + [("p2", False, 16), ("p2", False, 8), ("double", False, 32)]
+CASE_IDS = DESIGN_IDS + ["P2HT-B16", "P2HT-B8", "DoubleHT-B32"]
+
+
+@pytest.fixture(scope="module")
+def ws():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2509_16407_gb300 import build as b
+    b.build()
+    import paper_2509_16407_gb300 as ws
+    ws.lib()
+    return ws
+
+
+@pytest.mark.parametrize("op", ["insert", "add", "replace"])
+@pytest.mark.parametrize("copies", [1, 3])
+@pytest.mark.parametrize("log2", [7, 11, 16])
+@pytest.mark.parametrize("scheme,meta,B", CASES, ids=CASE_IDS)
+def test_build_from_nothing(ws, oracle_mod, scheme, meta, B, log2, copies, op):
+    t = ws.Table(1 << log2, scheme, meta, bucket_slots=B)
+    n = int((0.35 if B == 8 else 0.55) * (1 << log2))  # no insert may fail, whatever the interleaving
+    uniq = W.distinct_keys(4200 + log2, n)
+    keys = np.repeat(uniq, copies)[W.permutation(4300 + log2, n * copies)]
+    vals = W.mix13(keys) | np.uint64(1)  # one value per key: which copy wins does not show
+    got = host(t.upsert(dev(keys), dev(vals), op=op, return_status=True))
+    assert set(np.unique(got)) <= {ws.INSERTED, ws.FOUND}
+    assert (got == ws.INSERTED).sum() == n
+    first = np.unique(keys[got == ws.INSERTED])
+    assert first.size == n  # one INSERTED copy per key
+    with np.errstate(over="ignore"):
+        want = (W.mix13(uniq) | np.uint64(1)) * np.uint64(copies if op == "add" else 1)
+    v, st = t.query(dev(uniq), return_status=True)
+    assert (host(st) == ws.FOUND).all() and (host(v) == want).all()
+    check_layout(oracle_mod, t, n)
+    # the same keys after an erase: freed slots are claimed again
+    ev, es = t.erase(dev(uniq[::2]), return_values=True, return_status=True)
+    assert (host(es) == ws.FOUND).all() and (host(ev) == want[::2]).all()
+    again = host(t.upsert(dev(keys), dev(vals), op=op, return_status=True))
+    assert (again == ws.INSERTED).sum() == uniq[::2].size
+    assert t.count() == n
+    check_layout(oracle_mod, t, n)
+    assert t.last_error()["status"] == 0
+    t.close()
