@@ -235,6 +235,13 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
+// The sign bits of the two halves of a, then of b, each replicated over a byte.
+__device__ __forceinline__ u32 sign_bytes(u32 a, u32 b) {
+  u32 d;
+  asm("prmt.b32 %0, %1, %2, 0xfdb9;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+
 // Tag loads of 16, 8, 4 or 2 bytes (one lane's share of a 64-byte tag line).
 __device__ __forceinline__ void ld_tags16(const u16* p, u64& a, u64& b) {
   asm volatile(

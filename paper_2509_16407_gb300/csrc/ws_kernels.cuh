@@ -166,46 +166,63 @@ struct TileOps {
   // Lane snapshots (one lane per op; see the file comment)
   // ----------------------------------------------------------------------
   // Summary of a snapshot's 32 tags, packed in one word (it stays live
-  // across the candidate copy): bits 0-5 first tag equal to the key's (63:
-  // none), 6-11 number of such tags, 12-17 first free tag (always 63 here:
-  // see tag_free), 19 the bucket has an EMPTY slot, 20-25 occupancy as
+  // across the candidate copy): bits 0-5 a tag equal to the key's (63: none),
+  // 6-11 number of such tags, 12-17 first free tag (always 63 here: see
+  // tag_free), 19 the bucket has an EMPTY slot, 20-25 occupancy as
   // FILL_SHORTCUT - 1 (below the 3/4 threshold) or FILL_SHORTCUT (not below).
-  // Four tags per 64-bit word are tested at once: a field's bit 15 of
-  // zero16(x) is set exactly when the field of x is zero.  EMPTY slots form
-  // a suffix of a bucket (every claim takes the bucket's first free slot),
-  // so tag 31 tells whether the bucket has one; and in a table that never saw
-  // an erase (no tombstones: the only case the two-choice shortcut runs),
-  // occupancy is below 3/4 exactly when tag 3B/4 - 1 is EMPTY.
+  // EMPTY slots form a suffix of a bucket (every claim takes the bucket's
+  // first free slot), so tag 31 tells whether the bucket has one; and in a
+  // table that never saw an erase (no tombstones: the only case the two-choice
+  // shortcut runs), occupancy is below 3/4 exactly when tag 3B/4 - 1 is EMPTY.
   static constexpr u32 kTsNone = 63u;
-  __device__ static __forceinline__ u64 zero16(u64 x) {
-    constexpr u64 lo = 0x7fff7fff7fff7fffull, hi = 0x8000800080008000ull;
-    return ~(((x & lo) + lo) | x) & hi;  // (f & 0x7fff) + 0x7fff <= 0xfffe: no carry between fields
+
+  // Which of a snapshot's 32 tags, ANDed with `keep`, equal the tag k (both
+  // given twice in a word): bit 8 i + p of the result for tag 4 p + i.  Two
+  // tags per word: with x = tags ^ k, bit 15 of a half of
+  // ((x & 0x7fff7fff) + 0x7fff7fff) | x is clear exactly when the half of x is
+  // zero (the sum carries into no other half), and one byte permutation that
+  // replicates sign bits gathers the four answers of two words.  About 70
+  // instructions for a mask that gives any match, their number (one popc) and
+  // the first one, where testing 64-bit words and walking them again for the
+  // number took 60 to 200.  The metadata kernels are bound by instruction
+  // issue when L2 holds the table: 2^22-slot P2HT(M), 1M positive queries 45.5
+  // -> 36.4 us, 209,715 inserts 62 -> 52 us; 2^23-slot IcebergHT(M), 6.7M
+  // inserts 650 -> 540 us.
+  __device__ static __forceinline__ u32 tag_mask(const uint4 (&t)[4], u32 keep, u32 k) {
+    u32 m = 0;
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+      const u32 w0 = (p & 1) ? t[p / 2].z : t[p / 2].x, w1 = (p & 1) ? t[p / 2].w : t[p / 2].y;
+      const u32 x0 = (w0 & keep) ^ k, x1 = (w1 & keep) ^ k;
+      const u32 s0 = ((x0 & 0x7fff7fffu) + 0x7fff7fffu) | x0, s1 = ((x1 & 0x7fff7fffu) + 0x7fff7fffu) | x1;
+      m |= ~ptx::sign_bytes(s0, s1) & (0x01010101u << p);
+    }
+    return m;
   }
-  __device__ static __forceinline__ u64 tag_word(const PreWarp* pw, int j, int i) {
-    return reinterpret_cast<const u64*>(&pw->at(j, i >> 1))[i & 1];
+  // The lowest tag of a tag_mask (not 0).
+  __device__ static __forceinline__ u32 tag_first(u32 m) {
+    const u32 h = m | (m >> 16);
+    const u32 p = (u32)__ffs((int)((h | (h >> 8)) & 0xffu)) - 1u;
+    return 4u * p + (((u32)__ffs((int)((m >> p) & 0x01010101u)) - 1u) >> 3);
+  }
+  __device__ static __forceinline__ void tag_rows(const PreWarp* pw, int j, uint4 (&t)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) t[i] = *reinterpret_cast<const uint4*>(&pw->at(j, i));
   }
   __device__ static __forceinline__ u32 tag_scan(const PreWarp* pw, int j, u16 kt) {
-    const u64 k4 = (u64)kt * 0x0001000100010001ull;
-    u64 any = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) any |= zero16(tag_word(pw, j, i) ^ k4);
-    u32 first = kTsNone, nmatch = 0;
-    if (any) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const u64 me = zero16(tag_word(pw, j, i) ^ k4);
-        nmatch += (u32)__popcll(me);
-        if (first == kTsNone && me) first = 4u * i + (u32)(__ffsll((long long)me) >> 4) - 1u;
-      }
-    }
-    const u16* t = reinterpret_cast<const u16*>(&pw->at(j, 0));
-    const u32 empty = t[31] == TAG_EMPTY;
-    const u32 occ = (t[FILL_SHORTCUT - 1] == TAG_EMPTY) ? FILL_SHORTCUT - 1 : FILL_SHORTCUT;
-    return first | (nmatch << 6) | (kTsNone << 12) | (empty << 19) | (occ << 20);
+    uint4 t[4];
+    tag_rows(pw, j, t);
+    const u32 m = tag_mask(t, 0xffffffffu, (u32)kt * 0x00010001u);
+    const u32 bit = (u32)__ffs((int)m) - 1u;  // any match will do as the candidate
+    const u32 match = m ? 4u * (bit & 7u) + (bit >> 3) : kTsNone;
+    const u32 empty = (t[3].w >> 16) == TAG_EMPTY;
+    static_assert(!META || FILL_SHORTCUT == 24, "tag 23 is the upper half of word 11");
+    const u32 occ = (t[2].w >> 16) == TAG_EMPTY ? FILL_SHORTCUT - 1 : FILL_SHORTCUT;
+    return match | ((u32)__popc(m) << 6) | (kTsNone << 12) | (empty << 19) | (occ << 20);
   }
 
-  // Metadata second copy of a wave: the first slot of bucket b whose tag
-  // matches K, for op j.  Returns the snapshot's tag summary.
+  // Metadata second copy of a wave: a slot of bucket b whose tag matches K,
+  // for op j.  Returns the snapshot's tag summary.
   __device__ static __forceinline__ u32 preload_candidate(const TableView& tv, u64 K, u64 b0, PreWarp* pw, int j) {
     const u32 ts = tag_scan(pw, j, key_tag(K));
     const u32 q = ts & 63u;
@@ -1036,16 +1053,12 @@ struct TileOps {
   // in it (the tag summary leaves them out): the first free tag (EMPTY or
   // TOMB), whether it is EMPTY, and the exact occupancy.
   __device__ static __forceinline__ void tag_free(PreRef p, Snap& sn) {
-    u32 ffree = kTsNone, nfree = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const u64 mf = zero16(tag_word(p.w, p.j, i) & 0xfffefffefffefffeull);  // tag < 2
-      nfree += (u32)__popcll(mf);
-      if (ffree == kTsNone && mf) ffree = 4u * i + (u32)(__ffsll((long long)mf) >> 4) - 1u;
-    }
-    sn.occ = 32u - nfree;
-    sn.ffree = ffree == kTsNone ? -1 : (int)ffree;
-    sn.ffree_empty = ffree != kTsNone && p.tagrow(0)[ffree] == TAG_EMPTY;
+    uint4 t[4];
+    tag_rows(p.w, p.j, t);
+    const u32 m = tag_mask(t, 0xfffefffeu, 0u);  // tag < 2
+    sn.occ = 32u - (u32)__popc(m);
+    sn.ffree = m ? (int)tag_first(m) : -1;
+    sn.ffree_empty = m && p.tagrow(0)[sn.ffree] == TAG_EMPTY;
   }
 
   // Slot index and pair of the snapshot hit.
@@ -1333,7 +1346,7 @@ __device__ __forceinline__ void count_failure(const TableView& tv, u8 st) {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kChunkPasses = 4;  // 32-op chunks: lane passes of an insert whose lock or claim was lost before the tiles
-constexpr int kLaneRestarts = 2;  // streaming lane: restarts of an op after a lost CAS before the tiles
+constexpr int kLaneRestarts = 4;  // streaming lane: restarts of an op after a lost CAS before the tiles
 
 struct WarpSmem {
   u64 key[32], val[32], out[32], h1[32], h2[32];
@@ -1906,24 +1919,16 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           if (a.status_out) a.status_out[gi] = st;
           if (st >= ST_FULL) count_failure(tv, st);
           state = L_EMPTY;
-        } else if (r == -2 && kLaneLock && !locked &&
-                   Ops::lane_lock(tv, Ops::lock_of(tv, sm.h2[lane]))) {
-          // absent without the lock: now holding b_0's lock, follow the
-          // sequence again from b_0 and insert from what it reads
-          locked = true;
-          opk = Ops::LW_INSERT_LOCKED;
-          w = 0;
-          ls.ff_set = false;
-          ls.ff_idx = ls.ff_k = ls.ff_v = 0;
-          ls.occ0 = ls.occ1 = ls.cur_occ = ls.next_w = 0;
-          ls.f1_set = false;
-          ls.tsum = 0;
-          ls.f1_idx = ls.f1_k = ls.f1_v = 0;
-        } else if (r == -1 && !fresh && restarts < kLaneRestarts) {
-          // a lost CAS: the table moved under the snapshot (another claim
-          // or erase in this bucket).  Follow the sequence again from b_0
-          // -- its lines are in L2 now -- instead of handing the op to a
-          // tile; a held lock stays held.
+        } else if (((r == -2 && kLaneLock && !locked) || (r == -1 && !fresh)) && restarts < kLaneRestarts) {
+          // Absent without the lock: take it now, or -- its holder may be
+          // inserting this very key -- look again without it.  Or a lost
+          // claim: the table moved under the snapshot; a held lock stays held.
+          // Either way follow the sequence again from b_0 (its lines are in
+          // L2 now) instead of handing the op to a tile.
+          if (r == -2 && Ops::lane_lock(tv, Ops::lock_of(tv, sm.h2[lane]))) {
+            locked = true;
+            opk = Ops::LW_INSERT_LOCKED;
+          }
           ++restarts;
           fresh = true;
           w = 0;
