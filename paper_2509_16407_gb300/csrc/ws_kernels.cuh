@@ -1076,7 +1076,7 @@ struct TileOps {
   // Lane waves: the lane owning an op settles it bucket by bucket from
   // snapshots of the probe sequence (wave w holds bucket w of every op still
   // open), the same rules as the tile probe.  lane_wave returns 1 when the op
-  // is settled, 0 to go on to the next wave, -1 to hand it to the tile path
+  // is settled (`out`: an upsert's slot index), 0 to go on to the next wave, -1 to hand it to the tile path
   // (more than the snapshot can tell, or a lost CAS), and -2 when an upsert
   // probed without the lock has proven its key absent: it must now take b_0's
   // lock and read again before it may insert.
@@ -1124,6 +1124,7 @@ struct TileOps {
       }
       if (opk != LW_ERASE) {
         apply(tv, idx, op, V);
+        out = idx;
         st = ST_FOUND;
         return 1;
       }
@@ -1181,6 +1182,7 @@ struct TileOps {
       fresh = false;
       return -1;
     }
+    out = idx;
     ++dcount;
     st = ST_INSERTED;
     return 1;
@@ -1201,6 +1203,7 @@ struct TileOps {
       }
       if (opk != LW_ERASE) {
         apply(tv, idx, op, V);
+        out = idx;
         st = ST_FOUND;
         return 1;
       }
@@ -1308,6 +1311,7 @@ struct TileOps {
       fresh = false;
       return -1;
     }
+    out = fidx;
     if (got == 2) {  // another op of the call has just inserted K here
       apply(tv, fidx, op, V);
       st = ST_FOUND;
@@ -1354,6 +1358,76 @@ struct WarpSmem {
   u8 op[32], st[32], fresh[32], list[32];  // list: open ops of a bucket pass
   u64 in_key[32], in_val[32];  // streaming lanes, host inputs: op i's key / value in slot i % 32
   PreWarp pre;
+};
+
+// Keys that a block of an add / max / replace launch has met several times and
+// knows to be in the table: later upserts of such a key in the same block are
+// settled here -- a sum (or maximum) in shared memory, one atomic to the slot
+// when the block ends -- instead of reading the key's line and updating its
+// value again.  Skewed batches need it: one line of one L2 slice serves every
+// copy of a hot key, about 4.6 ns each (8M upsert-adds of Zipf(0.99) keys, 1M
+// distinct, 4.7% of them the first, into a 2^21-slot DoubleHT: 1744 us, with
+// this 292 us; nearly uniform keys take 250).  Sets of four ways: with one way
+// a key of 1% of the batch was kept out by a rarer one often enough to take
+// 670 us.  A key is admitted when an op that has just settled found its own
+// fingerprint still in `seen`, which keeps the last key of each of 256 hash
+// classes: frequent keys meet themselves there, keys of a uniform batch do not.
+// Within one call nothing removes an upserted key, so the ops settled here are
+// FOUND and any order of the call's adds (or maxima) gives the same sum; of
+// several replacements any may be the last, so the later ones can be dropped.
+struct HotKeys {
+  static constexpr int kKeys = 64, kWays = 4, kSeen = 256;
+  u64 key[kKeys], acc[kKeys], idx[kKeys];  // sets of kWays
+  u16 seen[kSeen];
+
+  __device__ __forceinline__ void clear() {
+    for (int i = threadIdx.x; i < kKeys; i += blockDim.x) key[i] = acc[i] = 0;
+    for (int i = threadIdx.x; i < kSeen; i += blockDim.x) seen[i] = 0;
+  }
+  __device__ static __forceinline__ int set_of(u64 h1) { return ((int)(h1 >> 40) & (kKeys / kWays - 1)) * kWays; }
+  // True when K is resident and (K, V) has been settled; else `twice` tells
+  // whether K was the last key seen in its class.
+  __device__ __forceinline__ bool settle(u64 h1, u64 K, u64 V, int op, bool& twice) {
+    const int e = set_of(h1);
+    int way = -1;
+#pragma unroll
+    for (int i = 0; i < kWays; ++i)
+      if (*reinterpret_cast<volatile u64*>(&key[e + i]) == K) way = i;
+    if (way >= 0) {
+      if (op == OP_ADD)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&acc[e + way]), V);
+      else if (op == OP_MAX)
+        atomicMax(reinterpret_cast<unsigned long long*>(&acc[e + way]), V);
+      return true;
+    }
+    volatile u16* s = &seen[(int)(h1 >> 46) & (kSeen - 1)];
+    const u16 f = (u16)(h1 >> 24) | 1u;
+    twice = *s == f;
+    *s = f;
+    return false;
+  }
+  __device__ __forceinline__ void admit(u64 h1, u64 K, u64 at) {
+    const int e = set_of(h1);
+    for (int i = 0; i < kWays; ++i) {
+      const u64 old = atomicCAS(reinterpret_cast<unsigned long long*>(&key[e + i]), 0ull, K);
+      if (old == 0ull) idx[e + i] = at;
+      if (old == 0ull || old == K) return;
+    }
+  }
+  // After every warp of the block is done.  The key is looked at again: in a
+  // batch that also erases it (outside the contract) the slot may be another's.
+  __device__ __forceinline__ void flush(const TableView& tv, int op) {
+    for (int i = threadIdx.x; i < kKeys; i += blockDim.x) {
+      if (!key[i] || !acc[i]) continue;
+      u64 k, v;
+      ptx::ld_slot(tv.slots + idx[i], k, v);
+      if (k != key[i]) continue;
+      if (op == OP_MAX)
+        ptx::red_max_u64(&tv.slots[idx[i]].val, acc[i]);
+      else
+        ptx::red_add_u64(&tv.slots[idx[i]].val, acc[i]);
+    }
+  }
 };
 
 enum { FLAG_SNAP = 1, FLAG_DONE = 2 };
@@ -1647,6 +1721,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
         const PreRef p{&sm.pre, lane};
         const int r =
             Ops::lane_wave(tv, p, K, V, op, opk, w, sm.bw[lane], ls, out, st, dcount, fresh, KIND != KIND_ERASE);
+        if (opk != Ops::LW_QUERY && opk != Ops::LW_ERASE) out = 0;
         if (r > 0) {
           done = true;
         } else if (r < 0) {
@@ -1742,12 +1817,13 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
                                            u64 begin, u64 end, WarpSmem& sm, int lane, u64* ticket = nullptr,
-                                           u64 share = 0, u64 warps = 1) {
+                                           u64 share = 0, u64 warps = 1, HotKeys* hot = nullptr) {
   using Ops = TileOps<SCHEME, META, B, T>;
   enum { L_EMPTY = 0, L_ACTIVE = 1, L_PARKED = 2 };
   constexpr int NT = 32 / T;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || Ops::kLines;
+  constexpr bool kHot = KIND == KIND_UPSERT;
   const u64 ks = a.key_stride ? a.key_stride : 1;
   const bool lane_path = (KIND != KIND_PROBE) && tv.preload;
   // a cap on the waves of one op (WS_OPT_LANE_WAVES); by default the whole sequence
@@ -1808,7 +1884,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         const u8 code = (KIND == KIND_MIXED) ? a.ops[gi] : 0;
         const u64 h1 = fmix64(K ^ tv.seed1), h2 = fmix64(K ^ tv.seed2);
         u8 st = ST_MISS;
-        bool settled = false;
+        bool settled = false, twice = false;
         op = upsert_op;
         opk = -1;
         if (KIND == KIND_UPSERT && (a.flags & BATCH_SKIP_SENTINELS) && is_sentinel(K)) {
@@ -1831,11 +1907,16 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
                 : kind == KIND_ERASE ? Ops::LW_ERASE
                 : (KIND == KIND_UPSERT && lockfree && SCHEME == SCHEME_DOUBLE) ? Ops::LW_INSERT_FREE
                                                                                  : Ops::LW_UPDATE_ONLY;
+          if (kHot && hot && hot->settle(h1, K, V, op, twice)) {
+            settled = true;
+            if (a.vals_out) a.vals_out[gi] = 0;
+            if (a.status_out) a.status_out[gi] = ST_FOUND;
+          }
         }
         if (!settled) {
           sm.key[lane] = K;
           sm.val[lane] = V;
-          sm.op[lane] = code;
+          sm.op[lane] = kHot ? (u8)twice : code;
           sm.h1[lane] = h1;
           sm.h2[lane] = h2;
           sm.out[lane] = gi;  // the op's index
@@ -1872,6 +1953,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         }
       }
       next += ncons;
+      // lanes whose ops were settled by HotKeys take more before the wave
+      if (kHot && hot && !ring && next < end && __popc(__ballot_sync(kAll, state == L_EMPTY)) >= 4) continue;
     }
     // 2. one wave: copy each active lane's current bucket, then settle
     const unsigned act = __ballot_sync(kAll, state == L_ACTIVE);
@@ -1914,6 +1997,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
                              KIND != KIND_ERASE);
         const bool wrote = r > 0 && st == ST_INSERTED;
         if (r > 0) {
+          if (kHot && hot && sm.op[lane] && st <= ST_INSERTED) hot->admit(sm.h1[lane], sm.key[lane], out);
+          if (opk != Ops::LW_QUERY && opk != Ops::LW_ERASE) out = 0;
           const u64 gi = sm.out[lane];
           if (a.vals_out) a.vals_out[gi] = out;
           if (a.status_out) a.status_out[gi] = st;
@@ -1996,13 +2081,21 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
 constexpr u64 kChunkGroup = 4;     // 32-op chunks a warp takes per ticket
 constexpr u64 kStreamShare = 256;  // ops a streaming warp takes per ticket
 
-template <int SCHEME, bool META, int B, int T, int KIND>
+// INS: an insert-if-unique call (KIND_UPSERT), a kernel of its own: it has no
+// use for HotKeys (keys of a build are new, and looking for repeated ones cost
+// DoubleHT inserts 2.5%), and on locking tables none for the streaming lanes.
+template <int SCHEME, bool META, int B, int T, int KIND, bool INS = false>
 __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchArgs a) {
+  constexpr bool kHot = KIND == KIND_UPSERT && !INS;
   __shared__ WarpSmem s_w[kWarps];
   __shared__ long long s_cnt;
+  __shared__ HotKeys s_hot;
+  HotKeys* hot = kHot ? &s_hot : nullptr;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_cnt = 0;
+  if (kHot) hot->clear();
   __syncthreads();
+  const int op = INS ? (int)OP_INSERT : a.op;
   const bool lockfree = (KIND == KIND_UPSERT);  // one call is one phase: no erase runs with it
   int dcount = 0;
   // Insert-if-unique calls on tables whose inserts lock (two-choice,
@@ -2015,7 +2108,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   // (measured at 2^28 slots: negative queries 2.56 ms in rounds vs 3.54 by
   // lines, positive queries 1.51 vs 1.31, upserts 1.87 vs 1.66).
   constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
-  const bool lock_bound = (KIND == KIND_UPSERT) && SCHEME != SCHEME_DOUBLE && a.op == OP_INSERT;
+  constexpr bool lock_bound = INS && SCHEME != SCHEME_DOUBLE;
   // (WS_OPT_STREAM = 2 streams them too, by lines: fewer bytes for hits near
   // the front of b_0, more dependent steps for misses.)
   const bool rounds = kRounds && (KIND == KIND_QUERY || KIND == KIND_ERASE) && tv.stream != 2;
@@ -2041,19 +2134,20 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
       const u64 left = (nchunks - c1) / (4 * warps);
       if (left < group) group = left < 1 ? 1 : left;
       for (u64 ch = c0; ch < c1; ++ch)
-        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, a.op, lockfree, ch * 32, s_w[w], lane);
+        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane);
     }
   } else {
     u64 share = (a.n / (4 * warps) + 31) / 32 * 32;
     share = share < 32 ? 32 : (share > kStreamShare ? kStreamShare : share);
-    dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, a.op, lockfree, 0, 0, s_w[w], lane, ticket, share,
-                                                    warps);
+    dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, 0, 0, s_w[w], lane, ticket, share,
+                                                    warps, hot);
   }
   if (KIND != KIND_QUERY && KIND != KIND_PROBE) {
     const int mine = __reduce_add_sync(0xffffffffu, dcount);
     if (lane == 0 && mine) atomicAdd((unsigned long long*)&s_cnt, (unsigned long long)(long long)mine);
   }
   __syncthreads();  // every warp of the block is done with the ticket
+  if (kHot) hot->flush(tv, op);
   if (threadIdx.x == 0) {
     if ((KIND != KIND_QUERY && KIND != KIND_PROBE) && s_cnt)
       atomicAdd((unsigned long long*)&tv.ctr->count, (unsigned long long)s_cnt);
@@ -2091,7 +2185,9 @@ template <int SCHEME, bool META, int B, int T>
 cudaError_t launch_cfg(const TableView& tv, const BatchArgs& a, int kind, cudaStream_t s, int num_sms) {
   switch (kind) {
     case KIND_QUERY: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_QUERY>>(tv, a, s, num_sms);
-    case KIND_UPSERT: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_UPSERT>>(tv, a, s, num_sms);
+    case KIND_UPSERT:
+      return a.op == OP_INSERT ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND_UPSERT, true>>(tv, a, s, num_sms)
+                               : launch_sized<batch_kernel<SCHEME, META, B, T, KIND_UPSERT>>(tv, a, s, num_sms);
     case KIND_ERASE: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_ERASE>>(tv, a, s, num_sms);
     case KIND_MIXED: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_MIXED>>(tv, a, s, num_sms);
     case KIND_PROBE: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_PROBE>>(tv, a, s, num_sms);
