@@ -45,7 +45,8 @@ struct Counters {
   u64 n_badkey;   // ops on sentinel keys / unknown op codes
   u64 ticket;     // work ticket of the running single-table launch
   u64 done;       // blocks of that launch that finished; the last one zeroes both
-  u64 pad[2];
+  u64 live;       // two-choice, iceberg: `count` when the last single-table upsert or insert launch ended
+  u64 pad;
 };
 
 // What a kernel needs of a table, passed by value.

@@ -376,6 +376,8 @@ struct TileOps {
           }
           if (c.ballot(k == KEY_EMPTY)) break;  // the rest of the bucket is EMPTY
         }
+        // never erased: the first EMPTY slot's index (see lane_wave)
+        if (tv.shortcut && hf[bi]) occ[bi] = (u32)(fi[bi] - b * B);
         if (bi == 0 && tv.shortcut && occ[0] < FILL_SHORTCUT) {
           decided0 = true;
           break;
@@ -407,6 +409,7 @@ struct TileOps {
           fi[gg] = c.shfl(si, src);
           fk[gg] = c.shfl(k, src);
           fv[gg] = c.shfl(v, src);
+          if (tv.shortcut) occ[gg] = (u32)(src - gg * B);
         }
       }
       if (nbk == 1) decided0 = true;
@@ -658,6 +661,7 @@ struct TileOps {
         hf[bi] = true;
         fi[bi] = b * 32 + (u64)q;
         ft[bi] = ((me >> q) & 1u) ? TAG_EMPTY : TAG_TOMB;
+        if (tv.shortcut) occ[bi] = (u32)q;  // never erased: see lane_wave
       }
       if (bi == 0 && tv.shortcut && occ[0] < FILL_SHORTCUT) {
         decided0 = true;
@@ -800,10 +804,10 @@ struct TileOps {
   // took 60 us with a new probe after each lost claim, 22 us with this.  (With
   // more lock bits and lane passes, 6.7M inserts into a 2^23-slot IcebergHT(M)
   // went from 1387 to 650 us, 209,715 into a 2^22-slot P2HT(M) from 145 to
-  // 62 us.)  holder: only this lane may insert K (it holds K's lock).  Returns
-  // 1 claimed, 2 the slot at idx holds K (plain tables), 0 lost.
+  // 62 us.)  Returns 1 claimed, 2 the slot at idx holds K (plain tables), 0
+  // lost.
   __device__ static __forceinline__ int lane_claim(const TableView& tv, u64& idx, u64 limit, u64 fk, u64 fv, u64 K,
-                                                   u64 V, bool holder) {
+                                                   u64 V) {
     for (;;) {
       if (META) {
         const u16 got = ptx::cas_tag(tv.tags + idx, (u16)fk, key_tag(K));
@@ -811,7 +815,7 @@ struct TileOps {
           ptx::st_slot_relaxed(tv.slots + idx, K, V);
           return 1;
         }
-        if (got == key_tag(K) && !holder) return 0;  // perhaps K itself, its pair not written yet
+        if (got == key_tag(K)) return 0;  // perhaps K itself, its pair not written yet
         if (fk != TAG_EMPTY) return 0;
       } else {
         u64 got;
@@ -925,7 +929,9 @@ struct TileOps {
     }
     u8 st = ST_TIMEOUT;
     for (int attempt = 0; attempt < 256; ++attempt) {
-      const Scan r = scan(tv, c, K, h1, h2, no_pre());
+      // LOCKFREE: lanes may claim slots without the lock (LW_INSERT_FRONT)
+      const Scan r = scan<LOCKFREE>(tv, c, K, h1, h2, no_pre());
+      if (r.stuck) break;
       if (r.found) {
         if (c.tl == 0) apply(tv, r.idx, op, V);
         st = ST_FOUND;
@@ -1084,7 +1090,18 @@ struct TileOps {
   // LW_INSERT_FREE: lock-free first-free insert (double hashing, no erase
   // in the launch).  LW_INSERT_LOCKED: the lane holds b_0's lock (or the
   // launch is bulk-synchronous), so its snapshots are authoritative for K.
-  enum { LW_QUERY = 0, LW_INSERT_FREE = 1, LW_UPDATE_ONLY = 2, LW_ERASE = 3, LW_INSERT_LOCKED = 4 };
+  // LW_INSERT_FRONT: two-choice and iceberg inserts while no lock is held, into
+  // tables that were never erased.  Where the scheme leaves no choice -- an
+  // iceberg key whose front bucket has an EMPTY slot, a two-choice key whose
+  // b_0 has an EMPTY slot below the 3/4 threshold -- every inserter of K goes
+  // for the first free slot of the same
+  // bucket until it is taken, as under double hashing, and the claim's CAS
+  // decides: slots only fill up during the launch, so an op that finds that
+  // part of the bucket taken without K knows that no claim of K in it can
+  // still succeed.  Only keys that must choose between two buckets need the
+  // lock.  A holder may meet such a claim, so a slot's tag may be K's before
+  // its pair is written (lanes: `unsure`; tiles wait for the pair).
+  enum { LW_QUERY = 0, LW_INSERT_FREE = 1, LW_UPDATE_ONLY = 2, LW_ERASE = 3, LW_INSERT_LOCKED = 4, LW_INSERT_FRONT = 5 };
   struct LaneState {
     bool ff_set;  // first free slot of the probe sequence seen so far
     u64 ff_idx, ff_k, ff_v;
@@ -1170,15 +1187,15 @@ struct TileOps {
       st = ST_MISS;
       return 1;
     }
-    if (opk != LW_INSERT_LOCKED) return -2;  // absent, and this op holds no lock
+    if (opk != LW_INSERT_LOCKED && !(opk == LW_INSERT_FRONT && c == 0 && tv.shortcut && ls.occ0 < FILL_SHORTCUT))
+      return -2;  // absent, and this op holds no lock
     const int ch = p2_choice(ls.occ0, ls.ff_set, ls.cur_occ, ls.f1_set, c == 1);
     if (ch < 0) {
       st = ST_FULL;
       return 1;
     }
     u64 idx = ch == 0 ? ls.ff_idx : ls.f1_idx;
-    if (lane_claim(tv, idx, claim_limit(idx), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V, true) !=
-        1) {
+    if (lane_claim(tv, idx, claim_limit(idx), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) != 1) {
       fresh = false;
       return -1;
     }
@@ -1226,8 +1243,13 @@ struct TileOps {
     // snapshot an EMPTY slot in it still settles the whole bucket (EMPTY
     // slots form a suffix of the bucket)
     if (!META && PRE_SLOTS < B && !sn.empty) return -1;
-    const bool ins = (opk == LW_INSERT_FREE || opk == LW_INSERT_LOCKED);
+    const bool ins =
+        opk == LW_INSERT_FREE || opk == LW_INSERT_LOCKED || (SCHEME != SCHEME_DOUBLE && opk == LW_INSERT_FRONT);
     if (META && ins) tag_free(p, sn);  // K is not here: this lane may claim a slot
+    // Never erased: the slots before the first EMPTY one are the taken ones.
+    // (A snapshot is copied in 16-byte pieces, so a count could include later
+    // slots taken after the piece that shows an EMPTY one was read.)
+    if (SCHEME == SCHEME_P2 && ins && tv.shortcut) sn.occ = sn.ffree >= 0 ? (u32)sn.ffree : (u32)B;
     if (SCHEME == SCHEME_P2 && w == 0) ls.occ0 = sn.occ;
     if (SCHEME == SCHEME_ICEBERG && w == 1) {
       ls.occ1 = sn.occ;
@@ -1263,6 +1285,9 @@ struct TileOps {
       return 1;
     }
     if (!ins) return -2;  // absent, and this op holds no lock
+    if (SCHEME != SCHEME_DOUBLE && opk == LW_INSERT_FRONT &&
+        !(w == 0 && tv.shortcut && (SCHEME == SCHEME_ICEBERG ? sn.empty : sn.occ < FILL_SHORTCUT)))
+      return -2;
     u64 fidx = ls.ff_idx, fk = ls.ff_k, fv = ls.ff_v;
     if (SCHEME == SCHEME_DOUBLE) {
       if (!sn.empty || !ls.ff_set) return -1;
@@ -1306,7 +1331,7 @@ struct TileOps {
         }
       }
     }
-    const int got = lane_claim(tv, fidx, claim_limit(fidx), fk, fv, K, V, opk == LW_INSERT_LOCKED);
+    const int got = lane_claim(tv, fidx, claim_limit(fidx), fk, fv, K, V);
     if (got == 0) {
       fresh = false;
       return -1;
@@ -1434,7 +1459,7 @@ enum { FLAG_SNAP = 1, FLAG_DONE = 2 };
 
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
-                                          u64 base, WarpSmem& sm, int lane) {
+                                          u64 base, WarpSmem& sm, int lane, bool lock_first = true) {
   using Ops = TileOps<SCHEME, META, B, T>;
   const u64 ks = a.key_stride ? a.key_stride : 1;
   const u64 gi = base + lane;
@@ -1480,6 +1505,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
         opk = Ops::LW_ERASE;
       else if (KIND == KIND_UPSERT && lockfree && SCHEME == SCHEME_DOUBLE)
         opk = Ops::LW_INSERT_FREE;
+      else if (KIND == KIND_UPSERT && lockfree && !(SCHEME == SCHEME_P2 && op == OP_INSERT && lock_first))
+        opk = Ops::LW_INSERT_FRONT;
       else
         opk = Ops::LW_UPDATE_ONLY;
     }
@@ -1499,7 +1526,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || kRounds;
   const u64 b0 = Ops::bucket(tv, h1, h2, 0), lk = Ops::lock_of(tv, h2);
   bool locked = false;
-  if (kLaneLock && lane_ok && !done && opk == Ops::LW_UPDATE_ONLY && (op == OP_INSERT || tv.phased)) {
+  if (kLaneLock && lane_ok && !done && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT) &&
+      ((op == OP_INSERT && lock_first) || tv.phased)) {
     locked = tv.phased || Ops::lane_lock(tv, lk);  // bulk-synchronous: no locks
     if (locked) opk = Ops::LW_INSERT_LOCKED;
   }
@@ -1567,7 +1595,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
             own_q = lane == j ? q : own_q;
           }
           if (own_q >= 0) {
-            occ = 32u - (u32)__popc(own_f);
+            // never erased: the first EMPTY slot's index (see lane_wave)
+            occ = !tv.shortcut ? 32u - (u32)__popc(own_f) : own_f ? (u32)__ffs(own_f) - 1u : 32u;
             if (own_k) {
               hs = __ffs(own_k) - 1;
               hv = sm.pre.flat(own_q, hs).val;
@@ -1618,15 +1647,15 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
             out = 0;
             st = ST_MISS;
             done = true;
-          } else if (opk == Ops::LW_INSERT_LOCKED) {
+          } else if (opk == Ops::LW_INSERT_LOCKED ||
+                     (opk == Ops::LW_INSERT_FRONT && c == 0 && tv.shortcut && occ < Ops::FILL_SHORTCUT)) {
             const int ch = Ops::p2_choice(occ0, f0 >= 0, occ, fs >= 0, c == 1);
             if (ch < 0) {
               st = ST_FULL;
               done = true;
             } else {
               u64 idx = ch == 0 ? b0 * 32 + (u64)f0 : bc * 32 + (u64)fs;
-              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K, V,
-                                  true) == 1) {
+              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K, V) == 1) {
                 ++dcount;
                 st = ST_INSERTED;
                 done = true;
@@ -1675,7 +1704,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
       run = run && again;
       if (!__any_sync(0xffffffffu, run)) break;
       if (run) {
-        if (!locked && opk == Ops::LW_UPDATE_ONLY) {
+        if (!locked && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT)) {
           locked = Ops::lane_lock(tv, lk);
           if (locked) opk = Ops::LW_INSERT_LOCKED;
         }
@@ -1727,7 +1756,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
         } else if (r < 0) {
           run = false;
           if ((r == -2 && kLaneLock && !locked) ||
-              (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE)))
+              (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE ||
+                          (SCHEME != SCHEME_DOUBLE && opk == Ops::LW_INSERT_FRONT))))
             again = true;  // absent without the lock, or a lost claim
           else
             lane_ok = false;
@@ -1817,7 +1847,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
                                            u64 begin, u64 end, WarpSmem& sm, int lane, u64* ticket = nullptr,
-                                           u64 share = 0, u64 warps = 1, HotKeys* hot = nullptr) {
+                                           u64 share = 0, u64 warps = 1, HotKeys* hot = nullptr,
+                                           bool lock_first = true) {
   using Ops = TileOps<SCHEME, META, B, T>;
   enum { L_EMPTY = 0, L_ACTIVE = 1, L_PARKED = 2 };
   constexpr int NT = 32 / T;
@@ -1905,8 +1936,9 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           }
           opk = kind == KIND_QUERY ? Ops::LW_QUERY
                 : kind == KIND_ERASE ? Ops::LW_ERASE
-                : (KIND == KIND_UPSERT && lockfree && SCHEME == SCHEME_DOUBLE) ? Ops::LW_INSERT_FREE
-                                                                                 : Ops::LW_UPDATE_ONLY;
+                : !(KIND == KIND_UPSERT && lockfree) ? Ops::LW_UPDATE_ONLY
+                : SCHEME == SCHEME_DOUBLE            ? Ops::LW_INSERT_FREE
+                                                     : Ops::LW_INSERT_FRONT;
           if (kHot && hot && hot->settle(h1, K, V, op, twice)) {
             settled = true;
             if (a.vals_out) a.vals_out[gi] = 0;
@@ -1933,7 +1965,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           if (!lane_path) {
             state = L_PARKED;
           } else {
-            if (kLaneLock && opk == Ops::LW_UPDATE_ONLY && (op == OP_INSERT || tv.phased)) {
+            if (kLaneLock && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT) &&
+                ((op == OP_INSERT && lock_first) || tv.phased)) {
               locked = tv.phased || Ops::lane_lock(tv, Ops::lock_of(tv, h2));
               if (locked) opk = Ops::LW_INSERT_LOCKED;
             }
@@ -2083,10 +2116,15 @@ constexpr u64 kStreamShare = 256;  // ops a streaming warp takes per ticket
 
 // INS: an insert-if-unique call (KIND_UPSERT), a kernel of its own: it has no
 // use for HotKeys (keys of a build are new, and looking for repeated ones cost
-// DoubleHT inserts 2.5%), and on locking tables none for the streaming lanes.
-template <int SCHEME, bool META, int B, int T, int KIND, bool INS = false>
+// DoubleHT inserts 2.5%).
+// PATH: how the launch is served, chosen by launch_path: streaming lanes,
+// 32-op chunks, or either, by the table's load (inserts that may lock).  A
+// kernel that holds both spills registers for the one that it does not run
+// (2^22-slot P2HT(M) step: 226 us with both in every kernel, 219 us).
+enum { PATH_EITHER = 0, PATH_STREAM = 1, PATH_CHUNK = 2 };
+template <int SCHEME, bool META, int B, int T, int KIND, bool INS, int PATH>
 __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchArgs a) {
-  constexpr bool kHot = KIND == KIND_UPSERT && !INS;
+  constexpr bool kHot = KIND == KIND_UPSERT && !INS && PATH == PATH_STREAM;
   __shared__ WarpSmem s_w[kWarps];
   __shared__ long long s_cnt;
   __shared__ HotKeys s_hot;
@@ -2098,20 +2136,26 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   const int op = INS ? (int)OP_INSERT : a.op;
   const bool lockfree = (KIND == KIND_UPSERT);  // one call is one phase: no erase runs with it
   int dcount = 0;
-  // Insert-if-unique calls on tables whose inserts lock (two-choice,
-  // iceberg) take a lock for almost every op; streaming would pay that
-  // acquire once per wave instead of once per 32-op chunk.  Plain
-  // two-choice tables with 32-slot buckets read whole buckets in 32-op
-  // chunks (rounds) for queries and erases too: a negative query or an
-  // erase of a late key needs most of both buckets, which rounds fetch in
-  // fewer dependent steps than streaming lanes reading a line per wave
-  // (measured at 2^28 slots: negative queries 2.56 ms in rounds vs 3.54 by
-  // lines, positive queries 1.51 vs 1.31, upserts 1.87 vs 1.66).
-  constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
-  constexpr bool lock_bound = INS && SCHEME != SCHEME_DOUBLE;
-  // (WS_OPT_STREAM = 2 streams them too, by lines: fewer bytes for hits near
-  // the front of b_0, more dependent steps for misses.)
-  const bool rounds = kRounds && (KIND == KIND_QUERY || KIND == KIND_ERASE) && tv.stream != 2;
+  // Insert-if-unique calls on two-choice and iceberg tables: while most keys
+  // go where the scheme leaves no choice they insert without the lock
+  // (LW_INSERT_FRONT), in streaming lanes; on fuller tables most keys need it,
+  // so each op takes it before its first probe, in 32-op chunks (streaming
+  // would pay the acquire once per wave instead of once per chunk).  The line
+  // is the load halfway through the call: 0.75 for iceberg, 0.6 for P2HT(M),
+  // 0.5 for P2HT, whose streaming lanes read a bucket line by line.  2^27
+  // slots, a tenth of them inserted at 0.4-0.5 / 0.5-0.6 / 0.6-0.7 / 0.7-0.8
+  // load, lock-free against lock first: IcebergHT(M) 1125 / 1164 / 1242 / 1523
+  // us against 1302 / 1329 / 1414 / 1460, P2HT(M) 1138 / 1169 / 1313 / 1667
+  // against 1312 / 1324 / 1316 / 1332, P2HT 1188 / 1871 / 3574 / 5951 against
+  // 1489 / 1604 / 1846 / 2261 (and 607 against 1452 into an empty table).
+  bool lock_first = true;
+  if (PATH == PATH_EITHER) {
+    const u64 slots = (tv.nb_mask + 1) * B;
+    // `live` is constant during the launch (`count` is not: a block that starts
+    // late must choose as the others did)
+    const u64 live = tv.ctr->live + a.n / 2;
+    lock_first = !tv.shortcut || live >= slots / 20 * (SCHEME == SCHEME_ICEBERG ? 15 : META ? 12 : 10);
+  }
   // Work comes from the launch's ticket: warps that draw long probe
   // sequences take less of it.  Shares shrink with the batch so that a small
   // launch still spreads over every warp (about four shares per warp, 32 to
@@ -2119,7 +2163,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   // towards the end of the launch (guided self-scheduling).
   u64* ticket = &tv.ctr->ticket;
   const u64 warps = (u64)gridDim.x * kWarps;
-  if (!tv.stream || lock_bound || rounds) {
+  if (PATH == PATH_CHUNK || (PATH == PATH_EITHER && lock_first)) {
     const u64 nchunks = (a.n + 31) / 32;
     u64 group = nchunks / (4 * warps);
     group = group < 1 ? 1 : (group > kChunkGroup ? kChunkGroup : group);
@@ -2134,13 +2178,14 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
       const u64 left = (nchunks - c1) / (4 * warps);
       if (left < group) group = left < 1 ? 1 : left;
       for (u64 ch = c0; ch < c1; ++ch)
-        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane);
+        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane,
+                                                         lock_first);
     }
   } else {
     u64 share = (a.n / (4 * warps) + 31) / 32 * 32;
     share = share < 32 ? 32 : (share > kStreamShare ? kStreamShare : share);
     dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, 0, 0, s_w[w], lane, ticket, share,
-                                                    warps, hot);
+                                                    warps, hot, lock_first);
   }
   if (KIND != KIND_QUERY && KIND != KIND_PROBE) {
     const int mine = __reduce_add_sync(0xffffffffu, dcount);
@@ -2152,11 +2197,14 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     if ((KIND != KIND_QUERY && KIND != KIND_PROBE) && s_cnt)
       atomicAdd((unsigned long long*)&tv.ctr->count, (unsigned long long)s_cnt);
     // the launch's last block returns the ticket to zero for the next launch
-    // on this table (launches on one table are stream-ordered)
+    // on this table (launches on one table are stream-ordered) and notes how
+    // full inserts have left it
+    constexpr bool kNote = KIND == KIND_UPSERT && SCHEME != SCHEME_DOUBLE;
     __threadfence();
     if (atomicAdd((unsigned long long*)&tv.ctr->done, 1ull) == (unsigned long long)gridDim.x - 1) {
       atomicExch((unsigned long long*)&tv.ctr->ticket, 0ull);
       atomicExch((unsigned long long*)&tv.ctr->done, 0ull);
+      if (kNote) tv.ctr->live = atomicAdd((unsigned long long*)&tv.ctr->count, 0ull);
     }
   }
 }
@@ -2181,16 +2229,32 @@ cudaError_t launch_sized(const TableView& tv, const BatchArgs& a, cudaStream_t s
   return cudaGetLastError();
 }
 
+// Streaming lanes unless WS_OPT_STREAM is 0.  Plain two-choice tables with
+// 32-slot buckets read whole buckets in 32-op chunks (rounds) for queries and
+// erases: a negative query or an erase of a late key needs most of both
+// buckets, which rounds fetch in fewer dependent steps than streaming lanes
+// reading a line per wave (measured at 2^28 slots: negative queries 2.56 ms in
+// rounds vs 3.54 by lines, positive queries 1.51 vs 1.31, upserts 1.87 vs
+// 1.66); WS_OPT_STREAM = 2 streams them too.
+template <int SCHEME, bool META, int B, int T, int KIND, bool INS = false>
+cudaError_t launch_path(const TableView& tv, const BatchArgs& a, cudaStream_t s, int num_sms) {
+  constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
+  constexpr int kStream = INS && SCHEME != SCHEME_DOUBLE ? PATH_EITHER : PATH_STREAM;
+  const bool rounds = kRounds && (KIND == KIND_QUERY || KIND == KIND_ERASE) && tv.stream != 2;
+  return !tv.stream || rounds ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, PATH_CHUNK>>(tv, a, s, num_sms)
+                              : launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, kStream>>(tv, a, s, num_sms);
+}
+
 template <int SCHEME, bool META, int B, int T>
 cudaError_t launch_cfg(const TableView& tv, const BatchArgs& a, int kind, cudaStream_t s, int num_sms) {
   switch (kind) {
-    case KIND_QUERY: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_QUERY>>(tv, a, s, num_sms);
+    case KIND_QUERY: return launch_path<SCHEME, META, B, T, KIND_QUERY>(tv, a, s, num_sms);
     case KIND_UPSERT:
-      return a.op == OP_INSERT ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND_UPSERT, true>>(tv, a, s, num_sms)
-                               : launch_sized<batch_kernel<SCHEME, META, B, T, KIND_UPSERT>>(tv, a, s, num_sms);
-    case KIND_ERASE: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_ERASE>>(tv, a, s, num_sms);
-    case KIND_MIXED: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_MIXED>>(tv, a, s, num_sms);
-    case KIND_PROBE: return launch_sized<batch_kernel<SCHEME, META, B, T, KIND_PROBE>>(tv, a, s, num_sms);
+      return a.op == OP_INSERT ? launch_path<SCHEME, META, B, T, KIND_UPSERT, true>(tv, a, s, num_sms)
+                               : launch_path<SCHEME, META, B, T, KIND_UPSERT>(tv, a, s, num_sms);
+    case KIND_ERASE: return launch_path<SCHEME, META, B, T, KIND_ERASE>(tv, a, s, num_sms);
+    case KIND_MIXED: return launch_path<SCHEME, META, B, T, KIND_MIXED>(tv, a, s, num_sms);
+    case KIND_PROBE: return launch_path<SCHEME, META, B, T, KIND_PROBE>(tv, a, s, num_sms);
   }
   return cudaErrorInvalidValue;
 }

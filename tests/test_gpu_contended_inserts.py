@@ -55,3 +55,30 @@ def test_build_from_nothing(ws, oracle_mod, scheme, meta, B, log2, copies, op):
     check_layout(oracle_mod, t, n)
     assert t.last_error()["status"] == 0
     t.close()
+
+
+@pytest.mark.parametrize("slices", [2, 9])
+@pytest.mark.parametrize("log2", [12, 17])
+@pytest.mark.parametrize("scheme,meta,B", [c for c in CASES if c[0] != "double"],
+                         ids=[i for i, c in zip(CASE_IDS, CASES) if c[0] != "double"])
+def test_fill_across_the_lock_line(ws, oracle_mod, scheme, meta, B, log2, slices):
+    """Filled to 0.8 in slices, so that calls insert lock-free, lock first and
+    on either side of the load where that changes; every key twice per call."""
+    t = ws.Table(1 << log2, scheme, meta, bucket_slots=B)
+    n = int((0.6 if B == 8 else 0.8) * (1 << log2))
+    uniq = W.distinct_keys(4400 + log2, n)
+    om = oracle_mod.OracleMap()
+    for i in range(slices):
+        part = uniq[i * n // slices:(i + 1) * n // slices]
+        keys = np.concatenate([part, part])[W.permutation(4500 + i, 2 * part.size)]
+        vals = W.mix13(keys)
+        st = host(t.insert(dev(keys), dev(vals), return_status=True))
+        om.insert(keys, vals)
+        assert (st == ws.INSERTED).sum() == part.size and (st == ws.FOUND).sum() == part.size
+        assert np.unique(keys[st == ws.INSERTED]).size == part.size
+    assert t.count() == n == om.count()
+    v, st = t.query(dev(uniq), return_status=True)
+    want, wst = om.query(uniq)
+    assert (host(v) == want).all() and (host(st) == wst).all()
+    check_layout(oracle_mod, t, n)
+    t.close()
