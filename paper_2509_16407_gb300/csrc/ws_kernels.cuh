@@ -51,6 +51,8 @@
 // WS_FAIL_TIMEOUT.  A tile waiting for a lock keeps re-probing lock-free and
 // finishes without the lock as soon as the key appears.
 #pragma once
+#include <cstddef>
+
 #include "ws_device.cuh"
 
 namespace ws {
@@ -827,12 +829,17 @@ struct TileOps {
       if (++idx >= limit) return 0;
     }
   }
-  // How far a claim may move on from slot idx: to the end of its bucket, but
-  // under two choices only while the bucket stays below the 3/4 threshold
-  // (beyond it the other bucket may be the less loaded one).
-  __device__ static __forceinline__ u64 claim_limit(u64 idx) {
+  // How far a claim may move on from slot idx.  Where the scheme leaves no
+  // choice, to the end of the bucket (two choices: to the 3/4 threshold).
+  // Between two buckets, while the chosen one -- `spare` slots emptier than
+  // the other when they were read, and one fuller with every lost claim -- is
+  // not the fuller one: going on to the end of the bucket left iceberg tables
+  // of 2^12 to 2^17 slots with 3 to 13 FULL keys at 0.95, where there were
+  // none.
+  __device__ static __forceinline__ u64 claim_limit(u64 idx, bool choice, u32 spare) {
     const u64 first = idx & ~(u64)(B - 1);
-    return first + (SCHEME == SCHEME_P2 ? (u64)FILL_SHORTCUT : (u64)B);
+    const u64 end = first + (SCHEME == SCHEME_P2 && !choice ? (u64)FILL_SHORTCUT : (u64)B);
+    return !choice || idx + 1 + spare > end ? end : idx + 1 + spare;
   }
 
   // ----------------------------------------------------------------------
@@ -1195,7 +1202,8 @@ struct TileOps {
       return 1;
     }
     u64 idx = ch == 0 ? ls.ff_idx : ls.f1_idx;
-    if (lane_claim(tv, idx, claim_limit(idx), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) != 1) {
+    const bool choice = ls.occ0 >= FILL_SHORTCUT;
+    if (lane_claim(tv, idx, claim_limit(idx, choice, 0), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) != 1) {
       fresh = false;
       return -1;
     }
@@ -1289,6 +1297,8 @@ struct TileOps {
         !(w == 0 && tv.shortcut && (SCHEME == SCHEME_ICEBERG ? sn.empty : sn.occ < FILL_SHORTCUT)))
       return -2;
     u64 fidx = ls.ff_idx, fk = ls.ff_k, fv = ls.ff_v;
+    bool choice = false;
+    u32 spare = 0;
     if (SCHEME == SCHEME_DOUBLE) {
       if (!sn.empty || !ls.ff_set) return -1;
     } else if (SCHEME == SCHEME_ICEBERG) {
@@ -1303,6 +1313,8 @@ struct TileOps {
           st = ST_FULL;
           return 1;
         }
+        choice = true;
+        spare = ch == 2 ? (ls.occ1 > sn.occ ? ls.occ1 - sn.occ : 0) : (sn.occ > ls.occ1 ? sn.occ - ls.occ1 : 0);
         if (ch == 1) {
           fidx = ls.f1_idx;
           fk = ls.f1_k;
@@ -1319,6 +1331,8 @@ struct TileOps {
         st = ST_FULL;
         return 1;
       }
+      choice = ls.occ0 >= FILL_SHORTCUT;
+      if (w > 0) spare = ch == 1 ? (ls.occ0 > sn.occ ? ls.occ0 - sn.occ : 0) : (sn.occ > ls.occ0 ? sn.occ - ls.occ0 : 0);
       if (ch == (int)w) {  // the free slot of this wave's bucket
         if (META) {
           fidx = bw * 32 + (u64)sn.ffree;
@@ -1331,7 +1345,7 @@ struct TileOps {
         }
       }
     }
-    const int got = lane_claim(tv, fidx, claim_limit(fidx), fk, fv, K, V);
+    const int got = lane_claim(tv, fidx, claim_limit(fidx, choice, spare), fk, fv, K, V);
     if (got == 0) {
       fresh = false;
       return -1;
@@ -1459,7 +1473,7 @@ enum { FLAG_SNAP = 1, FLAG_DONE = 2 };
 
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
-                                          u64 base, WarpSmem& sm, int lane, bool lock_first = true) {
+                                          u64 base, WarpSmem& sm, int lane) {
   using Ops = TileOps<SCHEME, META, B, T>;
   const u64 ks = a.key_stride ? a.key_stride : 1;
   const u64 gi = base + lane;
@@ -1505,8 +1519,6 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
         opk = Ops::LW_ERASE;
       else if (KIND == KIND_UPSERT && lockfree && SCHEME == SCHEME_DOUBLE)
         opk = Ops::LW_INSERT_FREE;
-      else if (KIND == KIND_UPSERT && lockfree && !(SCHEME == SCHEME_P2 && op == OP_INSERT && lock_first))
-        opk = Ops::LW_INSERT_FRONT;
       else
         opk = Ops::LW_UPDATE_ONLY;
     }
@@ -1526,8 +1538,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || kRounds;
   const u64 b0 = Ops::bucket(tv, h1, h2, 0), lk = Ops::lock_of(tv, h2);
   bool locked = false;
-  if (kLaneLock && lane_ok && !done && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT) &&
-      ((op == OP_INSERT && lock_first) || tv.phased)) {
+  if (kLaneLock && lane_ok && !done && opk == Ops::LW_UPDATE_ONLY && (op == OP_INSERT || tv.phased)) {
     locked = tv.phased || Ops::lane_lock(tv, lk);  // bulk-synchronous: no locks
     if (locked) opk = Ops::LW_INSERT_LOCKED;
   }
@@ -1595,8 +1606,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
             own_q = lane == j ? q : own_q;
           }
           if (own_q >= 0) {
-            // never erased: the first EMPTY slot's index (see lane_wave)
-            occ = !tv.shortcut ? 32u - (u32)__popc(own_f) : own_f ? (u32)__ffs(own_f) - 1u : 32u;
+            occ = 32u - (u32)__popc(own_f);
             if (own_k) {
               hs = __ffs(own_k) - 1;
               hv = sm.pre.flat(own_q, hs).val;
@@ -1647,15 +1657,16 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
             out = 0;
             st = ST_MISS;
             done = true;
-          } else if (opk == Ops::LW_INSERT_LOCKED ||
-                     (opk == Ops::LW_INSERT_FRONT && c == 0 && tv.shortcut && occ < Ops::FILL_SHORTCUT)) {
+          } else if (opk == Ops::LW_INSERT_LOCKED) {
             const int ch = Ops::p2_choice(occ0, f0 >= 0, occ, fs >= 0, c == 1);
             if (ch < 0) {
               st = ST_FULL;
               done = true;
             } else {
               u64 idx = ch == 0 ? b0 * 32 + (u64)f0 : bc * 32 + (u64)fs;
-              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K, V) == 1) {
+              const bool choice = occ0 >= Ops::FILL_SHORTCUT && c == 1;
+              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx, choice, 0), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K,
+                                  V) == 1) {
                 ++dcount;
                 st = ST_INSERTED;
                 done = true;
@@ -1704,7 +1715,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
       run = run && again;
       if (!__any_sync(0xffffffffu, run)) break;
       if (run) {
-        if (!locked && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT)) {
+        if (!locked && opk == Ops::LW_UPDATE_ONLY) {
           locked = Ops::lane_lock(tv, lk);
           if (locked) opk = Ops::LW_INSERT_LOCKED;
         }
@@ -1756,8 +1767,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
         } else if (r < 0) {
           run = false;
           if ((r == -2 && kLaneLock && !locked) ||
-              (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE ||
-                          (SCHEME != SCHEME_DOUBLE && opk == Ops::LW_INSERT_FRONT))))
+              (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE)))
             again = true;  // absent without the lock, or a lost claim
           else
             lane_ok = false;
@@ -1848,7 +1858,7 @@ template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
                                            u64 begin, u64 end, WarpSmem& sm, int lane, u64* ticket = nullptr,
                                            u64 share = 0, u64 warps = 1, HotKeys* hot = nullptr,
-                                           bool lock_first = true) {
+                                           bool front = false) {
   using Ops = TileOps<SCHEME, META, B, T>;
   enum { L_EMPTY = 0, L_ACTIVE = 1, L_PARKED = 2 };
   constexpr int NT = 32 / T;
@@ -1938,7 +1948,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
                 : kind == KIND_ERASE ? Ops::LW_ERASE
                 : !(KIND == KIND_UPSERT && lockfree) ? Ops::LW_UPDATE_ONLY
                 : SCHEME == SCHEME_DOUBLE            ? Ops::LW_INSERT_FREE
-                                                     : Ops::LW_INSERT_FRONT;
+                : front                              ? Ops::LW_INSERT_FRONT
+                                                     : Ops::LW_UPDATE_ONLY;
           if (kHot && hot && hot->settle(h1, K, V, op, twice)) {
             settled = true;
             if (a.vals_out) a.vals_out[gi] = 0;
@@ -1966,7 +1977,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
             state = L_PARKED;
           } else {
             if (kLaneLock && (opk == Ops::LW_UPDATE_ONLY || opk == Ops::LW_INSERT_FRONT) &&
-                ((op == OP_INSERT && lock_first) || tv.phased)) {
+                ((op == OP_INSERT && !front) || tv.phased)) {
               locked = tv.phased || Ops::lane_lock(tv, Ops::lock_of(tv, h2));
               if (locked) opk = Ops::LW_INSERT_LOCKED;
             }
@@ -2136,25 +2147,33 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   const int op = INS ? (int)OP_INSERT : a.op;
   const bool lockfree = (KIND == KIND_UPSERT);  // one call is one phase: no erase runs with it
   int dcount = 0;
-  // Insert-if-unique calls on two-choice and iceberg tables: while most keys
-  // go where the scheme leaves no choice they insert without the lock
-  // (LW_INSERT_FRONT), in streaming lanes; on fuller tables most keys need it,
-  // so each op takes it before its first probe, in 32-op chunks (streaming
-  // would pay the acquire once per wave instead of once per chunk).  The line
-  // is the load halfway through the call: 0.75 for iceberg, 0.6 for P2HT(M),
-  // 0.5 for P2HT, whose streaming lanes read a bucket line by line.  2^27
-  // slots, a tenth of them inserted at 0.4-0.5 / 0.5-0.6 / 0.6-0.7 / 0.7-0.8
-  // load, lock-free against lock first: IcebergHT(M) 1125 / 1164 / 1242 / 1523
-  // us against 1302 / 1329 / 1414 / 1460, P2HT(M) 1138 / 1169 / 1313 / 1667
-  // against 1312 / 1324 / 1316 / 1332, P2HT 1188 / 1871 / 3574 / 5951 against
-  // 1489 / 1604 / 1846 / 2261 (and 607 against 1452 into an empty table).
-  bool lock_first = true;
-  if (PATH == PATH_EITHER) {
-    const u64 slots = (tv.nb_mask + 1) * B;
-    // `live` is constant during the launch (`count` is not: a block that starts
-    // late must choose as the others did)
-    const u64 live = tv.ctr->live + a.n / 2;
-    lock_first = !tv.shortcut || live >= slots / 20 * (SCHEME == SCHEME_ICEBERG ? 15 : META ? 12 : 10);
+  // Two-choice and iceberg tables: whether inserts go without the lock where
+  // the scheme leaves no choice (`front`, see LW_INSERT_FRONT), in streaming
+  // lanes.  Otherwise add / max / replace lock once the key is proven absent,
+  // and insert-if-unique ops before their first probe, in 32-op chunks
+  // (streaming would pay the acquire once per wave instead of once per chunk).
+  // Two lines, on `live`, the load that the last launch noted (not `count`,
+  // which moves during the launch: a block that starts late must choose as the
+  // others did).  Speed, by the load halfway through the call: 0.75 for
+  // iceberg, 0.5 for P2HT, whose streaming lanes read a bucket line by line.
+  // 2^27 slots, a tenth of them inserted at 0.4-0.5 / 0.5-0.6 / 0.6-0.7 /
+  // 0.7-0.8 load, lock-free against lock first: IcebergHT(M) 1125 / 1164 / 1242
+  // / 1523 us against 1302 / 1329 / 1414 / 1460, P2HT(M) 1138 / 1169 / 1313 /
+  // 1667 against 1312 / 1324 / 1316 / 1332, P2HT 1188 / 1871 / 3574 / 5951
+  // against 1489 / 1604 / 1846 / 2261 (and 607 against 1452 into an empty
+  // table).  Balance, by the load at the end of the call: keys without a choice
+  // get in before keys in flight that have one, which costs two choices some of
+  // their evenness.  Filling 2^22 slots to 0.95 with the first part in that
+  // order (simulated) leaves 578 keys without a slot in 32-slot buckets for a
+  // first part of 0.45, 590 for 0.6, 678 for 0.7, 938 for 0.8, and 578 with
+  // none; for 16-slot buckets at 0.85 48, 64, 105, 227 and 47.
+  constexpr bool kFront = KIND == KIND_UPSERT && SCHEME != SCHEME_DOUBLE && PATH != PATH_CHUNK;
+  bool front = false;
+  if (kFront) {
+    const u64 slots = (tv.nb_mask + 1) * B, live = tv.ctr->live;
+    front = tv.shortcut && (SCHEME == SCHEME_ICEBERG
+                                ? live + a.n / 2 < slots / 4 * 3
+                                : live + a.n <= slots / 20 * (B == 32 ? 12 : 9) && (META || live + a.n / 2 < slots / 2));
   }
   // Work comes from the launch's ticket: warps that draw long probe
   // sequences take less of it.  Shares shrink with the batch so that a small
@@ -2163,7 +2182,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   // towards the end of the launch (guided self-scheduling).
   u64* ticket = &tv.ctr->ticket;
   const u64 warps = (u64)gridDim.x * kWarps;
-  if (PATH == PATH_CHUNK || (PATH == PATH_EITHER && lock_first)) {
+  if (PATH == PATH_CHUNK || (PATH == PATH_EITHER && !front)) {
     const u64 nchunks = (a.n + 31) / 32;
     u64 group = nchunks / (4 * warps);
     group = group < 1 ? 1 : (group > kChunkGroup ? kChunkGroup : group);
@@ -2178,14 +2197,13 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
       const u64 left = (nchunks - c1) / (4 * warps);
       if (left < group) group = left < 1 ? 1 : left;
       for (u64 ch = c0; ch < c1; ++ch)
-        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane,
-                                                         lock_first);
+        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane);
     }
   } else {
     u64 share = (a.n / (4 * warps) + 31) / 32 * 32;
     share = share < 32 ? 32 : (share > kStreamShare ? kStreamShare : share);
     dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, 0, 0, s_w[w], lane, ticket, share,
-                                                    warps, hot, lock_first);
+                                                    warps, hot, front);
   }
   if (KIND != KIND_QUERY && KIND != KIND_PROBE) {
     const int mine = __reduce_add_sync(0xffffffffu, dcount);

@@ -63,22 +63,34 @@ def test_build_from_nothing(ws, oracle_mod, scheme, meta, B, log2, copies, op):
                          ids=[i for i, c in zip(CASE_IDS, CASES) if c[0] != "double"])
 def test_fill_across_the_lock_line(ws, oracle_mod, scheme, meta, B, log2, slices):
     """Filled to 0.8 in slices, so that calls insert lock-free, lock first and
-    on either side of the load where that changes; every key twice per call."""
+    on either side of the load where that changes; every key twice per call.
+    8-slot buckets may report FULL at 0.6 (a few of 10^6 keys, whatever the
+    order): then both of the key's buckets must be full."""
     t = ws.Table(1 << log2, scheme, meta, bucket_slots=B)
     n = int((0.6 if B == 8 else 0.8) * (1 << log2))
     uniq = W.distinct_keys(4400 + log2, n)
     om = oracle_mod.OracleMap()
+    failed = []
     for i in range(slices):
         part = uniq[i * n // slices:(i + 1) * n // slices]
         keys = np.concatenate([part, part])[W.permutation(4500 + i, 2 * part.size)]
         vals = W.mix13(keys)
         st = host(t.insert(dev(keys), dev(vals), return_status=True))
-        om.insert(keys, vals)
-        assert (st == ws.INSERTED).sum() == part.size and (st == ws.FOUND).sum() == part.size
-        assert np.unique(keys[st == ws.INSERTED]).size == part.size
-    assert t.count() == n == om.count()
+        bad = np.unique(keys[st == ws.FAIL_FULL])
+        failed.append(bad)
+        ok = part.size - bad.size
+        om.insert(keys[~np.isin(keys, bad)], vals[~np.isin(keys, bad)])
+        assert (st == ws.INSERTED).sum() == ok and (st == ws.FOUND).sum() == ok
+        assert (st == ws.FAIL_FULL).sum() == 2 * bad.size
+        assert np.unique(keys[st == ws.INSERTED]).size == ok
+    failed = np.concatenate(failed)
+    assert failed.size <= (1e-4 * n if B == 8 else 0)
+    assert t.count() == n - failed.size == om.count()
     v, st = t.query(dev(uniq), return_status=True)
     want, wst = om.query(uniq)
     assert (host(v) == want).all() and (host(st) == wst).all()
-    check_layout(oracle_mod, t, n)
+    _, L = check_layout(oracle_mod, t, n - failed.size)
+    if failed.size:
+        assert oracle_mod.candidates_full(L["slots"], L["tags"], L["nb"], L["B"], L["scheme"], L["pmax"], L["seed1"],
+                                          L["seed2"], failed).all()
     t.close()
