@@ -1394,10 +1394,17 @@ constexpr int kLaneRestarts = 4;  // streaming lane: restarts of an op after a l
 struct WarpSmem {
   u64 key[32], val[32], out[32], h1[32], h2[32];
   u64 bw[32];  // bucket of each op in the current wave
-  u8 op[32], st[32], fresh[32], list[32];  // list: open ops of a bucket pass
+  u8 op[32], st[32], fresh[32];
+  union {
+    u8 list[32];                   // whole-bucket rounds: open ops of a bucket pass
+    struct { u64 base, share; };   // streaming lanes: where ticketed shares start, ops of the next one
+  };
   u64 in_key[32], in_val[32];  // streaming lanes, host inputs: op i's key / value in slot i % 32
   PreWarp pre;
 };
+// Off a 128-byte boundary the copies into `pre` cost the whole-bucket rounds
+// 1.5-4% (2^24 queries of a 2^28-slot P2HT: 1347 us against 1387).
+static_assert(offsetof(WarpSmem, pre) % 128 == 0 && sizeof(WarpSmem) % 128 == 0, "snapshot alignment");
 
 // Keys that a block of an add / max / replace launch has met several times and
 // knows to be in the table: later upserts of such a key in the same block are
@@ -1849,16 +1856,15 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 // no lane of the warp holds a bucket lock a tile might wait for.  Refill
 // pauses once enough ops are parked to fill the tiles.
 // -------------------------------------------------------------------------
-// Work shares: with `ticket` null the warp serves [begin, end); otherwise it
-// takes shares of up to `share` ops (a multiple of 32) from the launch's
-// ticket, which counts ops (begin / end unused), whenever its lanes run dry,
-// so warps whose ops probe long keep fewer ops and all finish close
-// together; `warps` is the launch's warp count.
+// Work shares: the warp serves [begin, end), and, unless `ticket` is null,
+// then takes shares of up to sm.share ops (a multiple of 32) of [sm.base, n)
+// from the launch's ticket whenever its lanes run dry, so warps whose ops
+// probe long keep fewer ops and all finish close together.  (What a warp needs
+// once per share lives in shared memory, not in registers.)
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs& a, int upsert_op, bool lockfree,
                                            u64 begin, u64 end, WarpSmem& sm, int lane, u64* ticket = nullptr,
-                                           u64 share = 0, u64 warps = 1, HotKeys* hot = nullptr,
-                                           bool front = false) {
+                                           HotKeys* hot = nullptr, bool front = false) {
   using Ops = TileOps<SCHEME, META, B, T>;
   enum { L_EMPTY = 0, L_ACTIVE = 1, L_PARKED = 2 };
   constexpr int NT = 32 / T;
@@ -1879,8 +1885,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
   typename Ops::LaneState ls;
   int dcount = 0, tile_d = 0;
   u64 next = begin;
-  bool exhausted = ticket == nullptr;  // no more shares to take
-  if (ticket) next = end = 0;
+  bool exhausted = ticket == nullptr || sm.base >= a.n;  // no more shares to take
   // Input ring (host inputs read in place): slot s of in_key / in_val holds
   // the op i with i % 32 == s among the 32 ops from `next` on (shares start
   // at multiples of 32).  Lane s copies its slot's op when the share begins
@@ -1888,22 +1893,28 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
   // inputs in shared memory: the copies complete during the wave between.
   const bool ring = (a.flags & BATCH_HOST_INPUTS) != 0 && ticket != nullptr;
   const bool want_v = (KIND == KIND_UPSERT || KIND == KIND_MIXED) && a.vals != nullptr;
+  if (ring && begin + (u64)lane < end) {
+    ptx::cp_async8(&sm.in_key[lane], a.keys + (begin + lane) * ks);
+    if (want_v) ptx::cp_async8(&sm.in_val[lane], a.vals + (begin + lane) * ks);
+  }
   for (;;) {
     // 1. refill: empty lanes take the next ops of the range, in lane order
     unsigned parked = __ballot_sync(kAll, state == L_PARKED);
     const unsigned empty = __ballot_sync(kAll, state == L_EMPTY);
     if (!exhausted && empty && next >= end) {  // the share is used up: take the next one
       u64 first = 0;
-      if (lane == 0) first = atomicAdd((unsigned long long*)ticket, (unsigned long long)share);
-      first = __shfl_sync(kAll, first, 0);
+      const u64 share = sm.share;
+      if (lane == 0) first = sm.base + atomicAdd((unsigned long long*)ticket, (unsigned long long)share);
+      first = __shfl_sync(kAll, first, 0);  // every lane has read sm.share
       if (first < a.n) {
         next = first;
         end = (a.n - first < share) ? a.n : first + share;
         // guided shares: once fewer than four shares per warp are left, take
         // a quarter per warp of what is left (a multiple of 32, at least 32),
         // so that the warps run dry together at the end of the launch
-        const u64 left = ((a.n - end) / (4 * warps) + 31) / 32 * 32;
-        if (left < share) share = left < 32 ? 32 : left;
+        const u64 left = ((a.n - end) / (4u * kWarps * gridDim.x) + 31) / 32 * 32;
+        if (lane == 0 && left < share) sm.share = left < 32 ? 32 : left;
+        __syncwarp();
         if (ring && first + (u64)lane < end) {
           ptx::cp_async8(&sm.in_key[lane], a.keys + (first + lane) * ks);
           if (want_v) ptx::cp_async8(&sm.in_val[lane], a.vals + (first + lane) * ks);
@@ -2175,35 +2186,58 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
                                 ? live + a.n / 2 < slots / 4 * 3
                                 : live + a.n <= slots / 20 * (B == 32 ? 12 : 9) && (META || live + a.n / 2 < slots / 2));
   }
-  // Work comes from the launch's ticket: warps that draw long probe
-  // sequences take less of it.  Shares shrink with the batch so that a small
-  // launch still spreads over every warp (about four shares per warp, 32 to
-  // kStreamShare ops each; one to kChunkGroup chunks), and shrink again
-  // towards the end of the launch (guided self-scheduling).
+  // Every warp starts on a share of its own: half of an equal part of the
+  // batch, kStreamShare ops at most (chunked launches beyond that many ops per
+  // warp start on the ticket: their first grabs are small against them).  The
+  // rest comes from the launch's ticket, so that warps that draw long probe
+  // sequences take less of it, in shares that shrink with the batch (about
+  // four per warp, 32 to kStreamShare ops; one to kChunkGroup chunks) and
+  // again towards the end of the launch (guided self-scheduling).  A launch of
+  // at most 32 ops per warp never touches the ticket.  With every share from
+  // the ticket the 4864 first grabs queued on one address before any probing,
+  // and a launch of 1M ops made 20,000 grabs: 1000 queries 6.0 us against 4.8,
+  // 2^22-slot P2HT(M) step 217 us against 205, 2^26-slot DoubleHT(M) step 1148
+  // us against 1140.
   u64* ticket = &tv.ctr->ticket;
-  const u64 warps = (u64)gridDim.x * kWarps;
+  const u64 warps = (u64)gridDim.x * kWarps, gw = (u64)blockIdx.x * kWarps + w;
+  bool tickets;  // launch-uniform
   if (PATH == PATH_CHUNK || (PATH == PATH_EITHER && !front)) {
     const u64 nchunks = (a.n + 31) / 32;
     u64 group = nchunks / (4 * warps);
     group = group < 1 ? 1 : (group > kChunkGroup ? kChunkGroup : group);
+    u64 first = nchunks / (2 * warps);
+    first = first < 1 ? 1 : (first > kStreamShare / 32 ? 0 : first);
+    const u64 base = warps * first;
+    tickets = base < nchunks;
+    u64 c0 = gw * first;
+    u64 c1 = c0 + first < nchunks ? c0 + first : nchunks;
     for (;;) {
-      u64 c0 = 0;
-      if (lane == 0) c0 = atomicAdd((unsigned long long*)ticket, (unsigned long long)group);
+      for (u64 ch = c0; ch < c1; ++ch)
+        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane);
+      if (!tickets) break;
+      if (lane == 0) c0 = base + atomicAdd((unsigned long long*)ticket, (unsigned long long)group);
       c0 = __shfl_sync(0xffffffffu, c0, 0);
       if (c0 >= nchunks) break;
-      const u64 c1 = (nchunks - c0 < group) ? nchunks : c0 + group;
+      c1 = (nchunks - c0 < group) ? nchunks : c0 + group;
       // guided: once fewer than four groups per warp are left, take a
       // quarter per warp of what is left (at least one chunk)
       const u64 left = (nchunks - c1) / (4 * warps);
       if (left < group) group = left < 1 ? 1 : left;
-      for (u64 ch = c0; ch < c1; ++ch)
-        dcount += warp_chunk<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, ch * 32, s_w[w], lane);
     }
   } else {
     u64 share = (a.n / (4 * warps) + 31) / 32 * 32;
     share = share < 32 ? 32 : (share > kStreamShare ? kStreamShare : share);
-    dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, 0, 0, s_w[w], lane, ticket, share,
-                                                    warps, hot, front);
+    u64 first = a.n / (2 * warps) / 32 * 32;
+    first = first < 32 ? 32 : (first > kStreamShare ? kStreamShare : first);
+    const u64 base = warps * first;
+    tickets = base < a.n;
+    const u64 begin = gw * first < a.n ? gw * first : a.n;
+    const u64 end = a.n - begin < first ? a.n : begin + first;
+    s_w[w].base = base;  // the same value on every lane
+    s_w[w].share = share;
+    __syncwarp();
+    dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, begin, end, s_w[w], lane, ticket, hot,
+                                                    front);
   }
   if (KIND != KIND_QUERY && KIND != KIND_PROBE) {
     const int mine = __reduce_add_sync(0xffffffffu, dcount);
@@ -2214,15 +2248,17 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   if (threadIdx.x == 0) {
     if ((KIND != KIND_QUERY && KIND != KIND_PROBE) && s_cnt)
       atomicAdd((unsigned long long*)&tv.ctr->count, (unsigned long long)s_cnt);
-    // the launch's last block returns the ticket to zero for the next launch
+    // The launch's last block returns the ticket to zero for the next launch
     // on this table (launches on one table are stream-ordered) and notes how
-    // full inserts have left it
+    // full inserts have left it.
     constexpr bool kNote = KIND == KIND_UPSERT && SCHEME != SCHEME_DOUBLE;
-    __threadfence();
-    if (atomicAdd((unsigned long long*)&tv.ctr->done, 1ull) == (unsigned long long)gridDim.x - 1) {
-      atomicExch((unsigned long long*)&tv.ctr->ticket, 0ull);
-      atomicExch((unsigned long long*)&tv.ctr->done, 0ull);
-      if (kNote) tv.ctr->live = atomicAdd((unsigned long long*)&tv.ctr->count, 0ull);
+    if (tickets || kNote) {
+      __threadfence();
+      if (atomicAdd((unsigned long long*)&tv.ctr->done, 1ull) == (unsigned long long)gridDim.x - 1) {
+        atomicExch((unsigned long long*)&tv.ctr->ticket, 0ull);
+        atomicExch((unsigned long long*)&tv.ctr->done, 0ull);
+        if (kNote) tv.ctr->live = atomicAdd((unsigned long long*)&tv.ctr->count, 0ull);
+      }
     }
   }
 }
