@@ -5,9 +5,10 @@
 // item into chunks of kMultiChunk ops and groups them by the item's table
 // configuration -- one entry of a fixed menu of compiled (scheme, metadata,
 // bucket slots, tile) combinations -- and op kind.  One persistent kernel per
-// group takes the group's chunks from a ticket counter (dynamic scheduling:
-// item sizes differ by four orders of magnitude); each warp serves a 256-op
-// share of a chunk with the lane and tile code of the single-table kernel.
+// group hands the group's chunks out in 256-op shares, one warp at a time, from
+// a ticket counter (dynamic scheduling: item sizes differ by four orders of
+// magnitude); a warp serves a share with the lane and tile code of the
+// single-table kernel.
 // A group's chunks come from an explicit list, or from prefix sums of the
 // chunk counts of a range of items (the no-allocation call, whose scratch has
 // a fixed size).  Each (menu entry, kind) is its own kernel in its own
@@ -18,7 +19,7 @@
 namespace ws {
 
 constexpr int kWarpShare = 256;                   // ops of a chunk per warp
-constexpr int kMultiChunk = kWarps * kWarpShare;  // ops per chunk = one block iteration
+constexpr int kMultiChunk = kWarps * kWarpShare;  // ops per chunk = kWarps shares
 
 struct MultiItem {
   TableView tv;

@@ -23,63 +23,59 @@ __device__ __forceinline__ int multi_share(const MultiItem& it, u64 begin, u64 e
   }
 }
 
+// Every warp works alone: its own descriptor, its own place in the queue of
+// 256-op shares (the first by its number, the rest from the ticket).  When a
+// block took 2048-op chunks together, its warps waited for the slowest of
+// eight shares, and for the ticket, chunk and descriptor reads before each
+// chunk: 1024 tables of 2^10 to 2^22 slots, 70M ops in four phases, took 2520
+// us, now 2257.
 template <int SCHEME, bool META, int B, int T, int KIND>
 __global__ void __launch_bounds__(kThreads, 4) multi_kernel(MultiGroup g) {
   __shared__ WarpSmem s_w[kWarps];
-  __shared__ u32 s_item;
-  __shared__ u64 s_start;
-  __shared__ int s_stop;
-  __shared__ __align__(16) MultiItem s_it;
+  __shared__ __align__(16) MultiItem s_it[kWarps];
   static_assert(sizeof(MultiItem) % 8 == 0, "item copy");
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const u32 warps = gridDim.x * kWarps;
+  const MultiItem& it = s_it[w];
   u32 cur_item = 0xffffffffu;
-  for (;;) {
-    if (threadIdx.x == 0) {
-      const u32 c = atomicAdd(g.ticket, 1u);
-      s_stop = c >= g.n_chunks;
-      if (!s_stop) {
-        if (g.chunks) {
-          const MultiChunk ch = g.chunks[c];
-          s_item = ch.item;
-          s_start = ch.start;
-        } else {
-          const u32 gc = g.prefix[g.i0] + c;
-          u32 lo = g.i0, hi = g.i1 - 1;  // largest item with prefix[item] <= gc
-          while (lo < hi) {
-            const u32 mid = (lo + hi + 1) / 2;
-            if (g.prefix[mid] <= gc)
-              lo = mid;
-            else
-              hi = mid - 1;
-          }
-          s_item = lo;
-          s_start = (u64)(gc - g.prefix[lo]) * kMultiChunk;
-        }
+  for (u32 unit = blockIdx.x * kWarps + w; unit / kWarps < g.n_chunks;) {  // warp-uniform
+    u32 item;
+    u64 begin;
+    if (g.chunks) {
+      const MultiChunk ch = g.chunks[unit / kWarps];
+      item = ch.item;
+      begin = ch.start;
+    } else {
+      const u32 gc = g.prefix[g.i0] + unit / kWarps;
+      u32 lo = g.i0, hi = g.i1 - 1;  // largest item with prefix[item] <= gc
+      while (lo < hi) {
+        const u32 mid = (lo + hi + 1) / 2;
+        if (g.prefix[mid] <= gc)
+          lo = mid;
+        else
+          hi = mid - 1;
+      }
+      item = lo;
+      begin = (u64)(gc - g.prefix[lo]) * kMultiChunk;
+    }
+    begin += (u64)(unit % kWarps) * kWarpShare;
+    if (item != cur_item) {  // stage the item descriptor once
+      const u64* src = reinterpret_cast<const u64*>(g.items + item);
+      u64* dst = reinterpret_cast<u64*>(&s_it[w]);
+      for (int q = lane; q < (int)(sizeof(MultiItem) / 8); q += 32) dst[q] = src[q];
+      cur_item = item;
+      __syncwarp();
+    }
+    if (begin < it.a.n) {
+      const int n_here = (int)(it.a.n - begin < (u64)kWarpShare ? it.a.n - begin : (u64)kWarpShare);
+      int d = multi_share<SCHEME, META, B, T, KIND>(it, begin, begin + n_here, s_w[w], lane);
+      if (KIND != KIND_QUERY) {
+        d = __reduce_add_sync(0xffffffffu, d);
+        if (lane == 0 && d) atomicAdd((unsigned long long*)&it.tv.ctr->count, (unsigned long long)(long long)d);
       }
     }
-    __syncthreads();
-    if (s_stop) break;
-    const u32 item = s_item;
-    const u64 start = s_start;
-    if (item != cur_item) {  // block-uniform: stage the item descriptor once
-      const u64* src = reinterpret_cast<const u64*>(g.items + item);
-      u64* dst = reinterpret_cast<u64*>(&s_it);
-      for (int q = threadIdx.x; q < (int)(sizeof(MultiItem) / 8); q += blockDim.x) dst[q] = src[q];
-      cur_item = item;
-    }
-    __syncthreads();
-    const MultiItem& it = s_it;
-    const u64 base = start + (u64)w * kWarpShare;
-    int d = 0;
-    if (base < it.a.n) {
-      const u64 end = (it.a.n - base < (u64)kWarpShare) ? it.a.n : base + kWarpShare;
-      d = multi_share<SCHEME, META, B, T, KIND>(it, base, end, s_w[w], lane);
-    }
-    if (KIND != KIND_QUERY) {
-      d = __reduce_add_sync(0xffffffffu, d);  // every lane reaches this: base is warp-uniform
-      if (lane == 0 && d) atomicAdd((unsigned long long*)&it.tv.ctr->count, (unsigned long long)(long long)d);
-    }
-    __syncthreads();  // s_it is rewritten by the next iteration
+    if (lane == 0) unit = warps + atomicAdd(g.ticket, 1u);
+    unit = __shfl_sync(0xffffffffu, unit, 0);  // every lane is done with s_it
   }
 }
 
