@@ -83,6 +83,14 @@ enum { PTR_NULL = 0, PTR_DEVICE = 1, PTR_HOST = 2, PTR_OTHER_DEVICE = 3 };
 // The device's view of page-locked, mapped host memory, or null (pageable
 // memory, or a pointer that is not host memory).
 void* mapped_host(const void* p);
+// Whether writing a result array in place, element by element, could overwrite
+// inputs not read yet: the ranges overlap and are not element for element the
+// same (an element's input is read before its result is written).
+inline bool crosses(const void* out, u64 out_elem, const void* in, u64 in_elem, u64 n) {
+  if (!out || !in || (out == in && out_elem == in_elem)) return false;
+  const uintptr_t o = reinterpret_cast<uintptr_t>(out), i = reinterpret_cast<uintptr_t>(in);
+  return o < i + n * in_elem && i < o + n * out_elem;
+}
 // Table constructor; with a non-null stream it allocates and clears on that
 // stream without synchronising the device.
 ws_status table_create(const ws_config* cfg, cudaStream_t stream, ws_table** out);

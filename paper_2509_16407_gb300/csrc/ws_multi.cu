@@ -12,6 +12,19 @@ cudaError_t launch_multi_5(int kind, const MultiGroup& g, cudaStream_t s, int nu
 cudaError_t launch_multi_6(int kind, const MultiGroup& g, cudaStream_t s, int num_sms);
 cudaError_t launch_multi_7(int kind, const MultiGroup& g, cudaStream_t s, int num_sms);
 
+namespace {
+__global__ void counts_kernel(const MultiItem* items, u32 n, u64* counts) {
+  const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) counts[i] = items[i].tv.ctr->count;
+}
+}  // namespace
+
+cudaError_t launch_counts(const MultiItem* items, u32 n, u64* counts, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  counts_kernel<<<(n + 127) / 128, 128, 0, s>>>(items, n, counts);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_multi(int cfg, int kind, const MultiGroup& g, cudaStream_t s, int num_sms) {
   switch (cfg) {
     case 0: return launch_multi_0(kind, g, s, num_sms);

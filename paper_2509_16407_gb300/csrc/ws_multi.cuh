@@ -30,6 +30,18 @@ struct MultiItem {
   int pad;
 };
 
+// Where a mixed item's ops live when they are page-locked host memory (device
+// views; keys null: they are in device memory, as the item says).  A warp then
+// copies a share's inputs to the item's device arrays before it serves the
+// share and the share's results back after it.
+struct HostOps {
+  const u64* keys;
+  const u64* vals;
+  const u8* ops;
+  u64* vals_out;
+  u8* status_out;
+};
+
 struct MultiChunk {
   u32 item;
   u32 pad;
@@ -46,6 +58,7 @@ struct MultiGroup {
   u32 i0, i1;
   u32 n_chunks;
   u32* ticket;  // zeroed before the launch
+  const HostOps* host;  // one per item, or null (mixed groups only)
 };
 
 // Menu of compiled configurations (scheme, metadata, bucket slots, tile).
@@ -72,5 +85,9 @@ inline int multi_menu_index(int scheme, bool meta, int B, int T) {
 // Runs group g on stream s with the kernel of menu entry `cfg` and op kind
 // `kind` (grid: resident blocks of all SMs, at most one block per chunk).
 cudaError_t launch_multi(int cfg, int kind, const MultiGroup& g, cudaStream_t s, int num_sms);
+
+// counts[i] = live keys of item i's table (counts: the device's view of
+// page-locked host memory), after the launches before it on the stream.
+cudaError_t launch_counts(const MultiItem* items, u32 n, u64* counts, cudaStream_t s);
 
 }  // namespace ws

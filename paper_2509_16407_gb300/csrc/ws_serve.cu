@@ -45,6 +45,7 @@ struct SReq {
   double t_submit = 0, t_start = 0;
   uint64_t n_write = 0;  // insert / upsert ops (growth estimate)
   bool has_erase = false;
+  ws::HostOps host = {};  // device views of its buffers when all are page-locked and mapped
 };
 
 struct STable {
@@ -54,6 +55,8 @@ struct STable {
   uint64_t live = 0;             // exact live count after the last finished request
 };
 
+constexpr size_t kItemBytes = sizeof(ws::MultiItem) + sizeof(ws::HostOps);
+
 struct Slot {
   cudaStream_t s = nullptr;
   cudaEvent_t done = nullptr;
@@ -62,12 +65,13 @@ struct Slot {
   u64* d_out = nullptr;
   u8* d_ops = nullptr;
   u8* d_st = nullptr;
-  ws::MultiItem* d_items = nullptr;
+  ws::MultiItem* d_items = nullptr;   // a launch's n descriptors, then their n HostOps
   ws::MultiChunk* d_chunks = nullptr;
   u32* d_ticket = nullptr;             // one work ticket per menu entry
-  ws::MultiItem* h_items = nullptr;   // pinned
+  ws::MultiItem* h_items = nullptr;   // pinned, as d_items
   ws::MultiChunk* h_chunks = nullptr; // pinned
   u64* h_counts = nullptr;            // pinned, one per request
+  u64* m_counts = nullptr;            // its device view
   std::vector<uint64_t> reqs;
   std::vector<uint32_t> tabs;
   std::vector<ws_table*> retire;
@@ -122,12 +126,13 @@ bool slot_alloc(Slot& sl, u64 cap, u64 max_items, u64 max_chunks) {
             cudaMalloc(&sl.d_keys, cap * 8) == cudaSuccess && cudaMalloc(&sl.d_vals, cap * 8) == cudaSuccess &&
             cudaMalloc(&sl.d_out, cap * 8) == cudaSuccess && cudaMalloc(&sl.d_ops, cap) == cudaSuccess &&
             cudaMalloc(&sl.d_st, cap) == cudaSuccess &&
-            cudaMalloc(&sl.d_items, max_items * sizeof(ws::MultiItem)) == cudaSuccess &&
+            cudaMalloc(&sl.d_items, max_items * kItemBytes) == cudaSuccess &&
             cudaMalloc(&sl.d_chunks, max_chunks * sizeof(ws::MultiChunk)) == cudaSuccess &&
             cudaMalloc(&sl.d_ticket, ws::kMultiMenu * sizeof(u32)) == cudaSuccess &&
-            cudaMallocHost(&sl.h_items, max_items * sizeof(ws::MultiItem)) == cudaSuccess &&
+            cudaMallocHost(&sl.h_items, max_items * kItemBytes) == cudaSuccess &&
             cudaMallocHost(&sl.h_chunks, max_chunks * sizeof(ws::MultiChunk)) == cudaSuccess &&
-            cudaMallocHost(&sl.h_counts, max_items * sizeof(u64)) == cudaSuccess;
+            cudaMallocHost(&sl.h_counts, max_items * sizeof(u64)) == cudaSuccess &&
+            cudaHostGetDevicePointer(reinterpret_cast<void**>(&sl.m_counts), sl.h_counts, 0) == cudaSuccess;
   if (!ok) cudaGetLastError();
   return ok;
 }
@@ -217,6 +222,7 @@ bool launch_slot(ws_server* sv, Slot& sl) {
   u64 off = 0, nchunks = 0;
   bool ok = true;
   std::vector<int> fallback;
+  ws::HostOps* h_host = reinterpret_cast<ws::HostOps*>(sl.h_items + sl.reqs.size());
   for (size_t i = 0; i < sl.reqs.size() && ok; ++i) {
     SReq& q = sv->reqs[sl.reqs[i]];
     q.t_start = t0;
@@ -226,18 +232,22 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     ws_table* t = T.t;
     if (q.has_erase) t->never_erased = 0;
     const u64 n = q.r.n;
-    ok = cudaMemcpyAsync(sl.d_keys + off, q.r.keys, n * 8, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         cudaMemcpyAsync(sl.d_ops + off, q.r.ops, n, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-         (q.r.vals ? cudaMemcpyAsync(sl.d_vals + off, q.r.vals, n * 8, cudaMemcpyHostToDevice, s)
-                   : cudaMemsetAsync(sl.d_vals + off, 0, n * 8, s)) == cudaSuccess;
     ws::MultiItem& m = sl.h_items[i];
     std::memset(&m, 0, sizeof(m));
     m.tv = t->tv;
     m.tv.shortcut = t->never_erased;
-    m.a = ws::BatchArgs{sl.d_keys + off, sl.d_vals + off, sl.d_ops + off, sl.d_out + off, sl.d_st + off, n, 0, 1, 0};
+    m.a = ws::BatchArgs{sl.d_keys + off, q.r.vals ? sl.d_vals + off : nullptr, sl.d_ops + off, sl.d_out + off,
+                        sl.d_st + off, n, 0, 1, 0};
     m.kind = ws::KIND_MIXED;
     m.cfg = sv->cfg.plain ? -1 : ws::multi_menu_index(t->scheme, t->meta != 0, (int)t->B, t->T);
     if (m.cfg < 0) fallback.push_back((int)i);
+    // page-locked requests are copied in and out by the kernel's own warps
+    h_host[i] = m.cfg >= 0 ? q.host : ws::HostOps{};
+    if (!h_host[i].keys)
+      ok = cudaMemcpyAsync(sl.d_keys + off, q.r.keys, n * 8, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+           cudaMemcpyAsync(sl.d_ops + off, q.r.ops, n, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+           (!q.r.vals ||
+            cudaMemcpyAsync(sl.d_vals + off, q.r.vals, n * 8, cudaMemcpyHostToDevice, s) == cudaSuccess);
     off += n;
   }
   // chunks grouped by menu entry (every request is a mixed batch): one
@@ -257,16 +267,17 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     }
   }
   group_off[ws::kMultiMenu] = nchunks;
+  if (ok)
+    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * kItemBytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
   if (ok && nchunks) {
-    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * sizeof(ws::MultiItem), cudaMemcpyHostToDevice,
-                         s) == cudaSuccess &&
-         cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
+    ok = cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
              cudaSuccess &&
          cudaMemsetAsync(sl.d_ticket, 0, ws::kMultiMenu * sizeof(u32), s) == cudaSuccess;
     for (int cfg = 0; cfg < ws::kMultiMenu && ok; ++cfg) {
       const u64 n_c = group_off[cfg + 1] - group_off[cfg];
       if (!n_c) continue;
-      ws::MultiGroup g{sl.d_items, sl.d_chunks + group_off[cfg], nullptr, 0, 0, (u32)n_c, sl.d_ticket + cfg};
+      ws::MultiGroup g{sl.d_items, sl.d_chunks + group_off[cfg], nullptr, 0, 0, (u32)n_c, sl.d_ticket + cfg,
+                       reinterpret_cast<const ws::HostOps*>(sl.d_items + sl.reqs.size())};
       ok = ws::launch_multi(cfg, ws::KIND_MIXED, g, s, sv->num_sms) == cudaSuccess;
     }
   }
@@ -278,15 +289,15 @@ bool launch_slot(ws_server* sv, Slot& sl) {
   for (size_t i = 0; i < sl.reqs.size() && ok; ++i) {
     SReq& q = sv->reqs[sl.reqs[i]];
     const u64 n = q.r.n;
-    if (q.r.vals_out)
+    const bool copied = h_host[i].keys != nullptr;
+    if (q.r.vals_out && !copied)
       ok = cudaMemcpyAsync(q.r.vals_out, sl.d_out + off, n * 8, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    if (ok && q.r.status_out)
+    if (ok && q.r.status_out && !copied)
       ok = cudaMemcpyAsync(q.r.status_out, sl.d_st + off, n, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    ws_table* t = sv->tables[sl.tabs[i]].t;
-    if (ok) ok = cudaMemcpyAsync(&sl.h_counts[i], &t->tv.ctr->count, 8, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-    t->last_stream = s;
+    sv->tables[sl.tabs[i]].t->last_stream = s;
     off += n;
   }
+  if (ok) ok = ws::launch_counts(sl.d_items, (u32)sl.reqs.size(), sl.m_counts, s) == cudaSuccess;
   if (ok) ok = cudaEventRecord(sl.done, s) == cudaSuccess;
   if (!ok) {
     note_cuda(cudaGetLastError(), "server launch");
@@ -330,6 +341,25 @@ void wake_worker(ws_server* sv) {
   sv->cv_in.notify_one();
 }
 
+// Device views of a request's buffers, or keys == nullptr when one of them is
+// not page-locked and mapped, or results overlap inputs other than their own.
+ws::HostOps host_ops(const ws_request& r) {
+  ws::HostOps h = {};
+  const u64 n = r.n;
+  if (n == 0 || crosses(r.vals_out, 8, r.keys, 8, n) || crosses(r.vals_out, 8, r.vals, 8, n) ||
+      crosses(r.vals_out, 8, r.ops, 1, n) || crosses(r.status_out, 1, r.keys, 8, n) ||
+      crosses(r.status_out, 1, r.vals, 8, n) || crosses(r.status_out, 1, r.ops, 1, n) ||
+      crosses(r.status_out, 1, r.vals_out, 8, n))
+    return h;
+  h.vals = static_cast<const u64*>(mapped_host(r.vals));
+  h.ops = static_cast<const u8*>(mapped_host(r.ops));
+  h.vals_out = static_cast<u64*>(mapped_host(r.vals_out));
+  h.status_out = static_cast<u8*>(mapped_host(r.status_out));
+  if (h.ops && (h.vals || !r.vals) && (h.vals_out || !r.vals_out) && (h.status_out || !r.status_out))
+    h.keys = static_cast<const u64*>(mapped_host(r.keys));
+  return h;
+}
+
 // Moves submitted requests into the per-table queues (worker, `mu` held);
 // counts each request's writes (growth estimate) and erases here, off the
 // submitting thread.
@@ -346,6 +376,7 @@ void take_inbox(ws_server* sv) {
       q.n_write += (o >= WS_MX_INSERT && o <= WS_MX_REPLACE) ? 1 : 0;
       q.has_erase |= (o == WS_MX_ERASE);
     }
+    q.host = host_ops(q.r);
     sv->tables[q.r.table].pending.push_back(q.id);
     sv->reqs.push_back(q);  // ids are handed out in inbox order: index == id
   }
