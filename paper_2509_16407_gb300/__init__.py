@@ -50,8 +50,15 @@ def _torch():
     return torch
 
 
+_TENSOR_TYPE = {np.ndarray: False}  # argument types met so far: the name test costs 0.3 us
+
+
 def _is_tensor(x):
-    return type(x).__module__.startswith("torch")
+    t = type(x)
+    r = _TENSOR_TYPE.get(t)
+    if r is None:
+        r = _TENSOR_TYPE[t] = t.__module__.startswith("torch")
+    return r
 
 
 def _ptr(x, itemsize=None):
@@ -131,6 +138,10 @@ class Table:
     def _stream(self, stream):
         if stream is None:
             torch = _torch()
+            # a small query is host-bound (1000 keys: 18 us a call, of which 4
+            # went into the device check and a Stream object; 14 with the handle)
+            if torch.cuda.is_initialized():
+                return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(self.device))
             if torch.cuda.is_available():
                 return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
             return None
