@@ -1388,7 +1388,10 @@ __device__ __forceinline__ void count_failure(const TableView& tv, u8 st) {
 // -------------------------------------------------------------------------
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kChunkPasses = 4;  // 32-op chunks: lane passes of an insert whose lock or claim was lost before the tiles
+// 32-op chunks: lane passes of an insert whose lock or claim was lost before the
+// tiles take it (13,107 inserts into a 2^18-slot P2HT at 0.8 load: 138 us with 2
+// passes, 64 with 4, 57 with 8; large tables do not care).
+constexpr int kChunkPasses = 8;
 constexpr int kLaneRestarts = 4;  // streaming lane: restarts of an op after a lost CAS before the tiles
 
 struct WarpSmem {
