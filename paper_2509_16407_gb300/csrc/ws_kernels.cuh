@@ -1089,13 +1089,14 @@ struct TileOps {
   // Lane waves: the lane owning an op settles it bucket by bucket from
   // snapshots of the probe sequence (wave w holds bucket w of every op still
   // open), the same rules as the tile probe.  lane_wave returns 1 when the op
-  // is settled (`out`: an upsert's slot index), 0 to go on to the next wave, -1 to hand it to the tile path
-  // (more than the snapshot can tell, or a lost CAS), and -2 when an upsert
-  // probed without the lock has proven its key absent: it must now take b_0's
-  // lock and read again before it may insert.
+  // is settled (`out`: an upsert's slot index), 0 to go on to the next wave,
+  // -1 when the snapshot cannot tell or a claim was lost (read again, or hand
+  // the op to the tiles), and -2 when an upsert that probed without the lock
+  // has proven its key absent: it must now take the key's lock and read again
+  // before it may insert.
   // ----------------------------------------------------------------------
   // LW_INSERT_FREE: lock-free first-free insert (double hashing, no erase
-  // in the launch).  LW_INSERT_LOCKED: the lane holds b_0's lock (or the
+  // in the launch).  LW_INSERT_LOCKED: the lane holds K's lock (or the
   // launch is bulk-synchronous), so its snapshots are authoritative for K.
   // LW_INSERT_FRONT: two-choice and iceberg inserts while no lock is held, into
   // tables that were never erased.  Where the scheme leaves no choice -- an
@@ -1324,7 +1325,7 @@ struct TileOps {
         }
       }
     } else {
-      // K is absent from its buckets and the lane holds b_0's lock: place it
+      // K is absent from its buckets and the lane may insert it: place it
       const bool free0 = (w == 0) ? sn.ffree >= 0 : ls.ff_set;
       const int ch = p2_choice(ls.occ0, free0, sn.occ, sn.ffree >= 0, w > 0);
       if (ch < 0) {
@@ -1375,7 +1376,7 @@ __device__ __forceinline__ void count_failure(const TableView& tv, u8 st) {
 //  1. Stage: lane j loads op j's key (value, op code) with coalesced loads and
 //     hashes it once; keys and hashes go to shared memory.
 //  2. Lock: an op that may have to insert under the lock (two-choice
-//     inserts, mixed batches) takes b_0's lock from its lane, one attempt.
+//     inserts, mixed batches) takes its key's lock from its lane, one attempt.
 //  3. Lane path: wave w copies bucket w of every open op into shared memory
 //     (cp.async; four ops' 128-byte lines per instruction, so each copy
 //     instruction is coalesced; with metadata the 64-byte tag line, then the
@@ -1539,12 +1540,12 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   // of first-line snapshots (below)
   constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
   // An insert-if-unique op that may insert under the lock (its key is most
-  // likely new) takes b_0's lock from its own lane, one attempt, before its
+  // likely new) takes its key's lock from its own lane, one attempt, before its
   // first copy; the lane's reads after it are then authoritative for K (only
-  // holders of b_0's lock insert K).  Add / max / replace probe lock-free
-  // first: a present key -- a hot Zipf key above all -- needs no lock, and an
-  // absent one goes to the tiles, which lock and rescan.  A lane that misses
-  // the lock also leaves absent keys to the tiles, which wait for it.
+  // holders of that lock insert K).  Add / max / replace probe lock-free
+  // first: a present key -- a hot Zipf key above all -- needs no lock.  An op
+  // that proved its key absent without the lock tries for it before its next
+  // pass (kChunkPasses).
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || kRounds;
   const u64 b0 = Ops::bucket(tv, h1, h2, 0), lk = Ops::lock_of(tv, h2);
   bool locked = false;
@@ -1856,8 +1857,9 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 // the lane path cannot settle (a lost CAS, an unsure tag match, an insert
 // without the lock, the probe-count kernel) are parked and served by the
 // cooperative tiles, which run only when no lane of the warp is active -- so
-// no lane of the warp holds a bucket lock a tile might wait for.  Refill
-// pauses once enough ops are parked to fill the tiles.
+// no lane of the warp holds a lock a tile might wait for.  An op that lost a
+// claim, or proved its key absent without the lock, first starts over in its
+// lane (kLaneRestarts).  Refill pauses once enough ops are parked to fill the tiles.
 // -------------------------------------------------------------------------
 // Work shares: the warp serves [begin, end), and, unless `ticket` is null,
 // then takes shares of up to sm.share ops (a multiple of 32) of [sm.base, n)
