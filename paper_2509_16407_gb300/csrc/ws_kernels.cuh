@@ -1401,7 +1401,10 @@ struct WarpSmem {
   u8 op[32], st[32], fresh[32];
   union {
     u8 list[32];                   // whole-bucket rounds: open ops of a bucket pass
-    struct { u64 base, share; };   // streaming lanes: where ticketed shares start, ops of the next one
+    struct {                       // streaming lanes:
+      u64 base, share;             // where ticketed shares start, ops of the next one
+      u32 hot_on;                  // mixed: the warp looks for frequent keys in this share
+    };
   };
   u64 in_key[32], in_val[32];  // streaming lanes, host inputs: op i's key / value in slot i % 32
   PreWarp pre;
@@ -1410,7 +1413,7 @@ struct WarpSmem {
 // 1.5-4% (2^24 queries of a 2^28-slot P2HT: 1347 us against 1387).
 static_assert(offsetof(WarpSmem, pre) % 128 == 0 && sizeof(WarpSmem) % 128 == 0, "snapshot alignment");
 
-// Keys that a block of an add / max / replace launch has met several times and
+// Keys that a block of an upsert or mixed launch has met several times and
 // knows to be in the table: later upserts of such a key in the same block are
 // settled here -- a sum (or maximum) in shared memory, one atomic to the slot
 // when the block ends -- instead of reading the key's line and updating its
@@ -1429,8 +1432,10 @@ struct HotKeys {
   static constexpr int kKeys = 64, kWays = 4, kSeen = 256;
   u64 key[kKeys], acc[kKeys], idx[kKeys];  // sets of kWays
   u16 seen[kSeen];
+  u32 hits, looked;  // mixed: ops settled here, ops of the shares that looked
 
   __device__ __forceinline__ void clear() {
+    if (threadIdx.x == 0) hits = looked = 0;
     for (int i = threadIdx.x; i < kKeys; i += blockDim.x) key[i] = acc[i] = 0;
     for (int i = threadIdx.x; i < kSeen; i += blockDim.x) seen[i] = 0;
   }
@@ -1465,7 +1470,8 @@ struct HotKeys {
     }
   }
   // After every warp of the block is done.  The key is looked at again: in a
-  // batch that also erases it (outside the contract) the slot may be another's.
+  // mixed batch that also erases it (outside the contract) the slot may be
+  // another's.
   __device__ __forceinline__ void flush(const TableView& tv, int op) {
     for (int i = threadIdx.x; i < kKeys; i += blockDim.x) {
       if (!key[i] || !acc[i]) continue;
@@ -1875,7 +1881,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
   constexpr int NT = 32 / T;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || Ops::kLines;
-  constexpr bool kHot = KIND == KIND_UPSERT;
+  constexpr bool kHot = KIND == KIND_UPSERT || KIND == KIND_MIXED;
+  constexpr u8 kTwice = 0x80;  // in sm.op: the op's key is frequent
   const u64 ks = a.key_stride ? a.key_stride : 1;
   const bool lane_path = (KIND != KIND_PROBE) && tv.preload;
   // a cap on the waves of one op (WS_OPT_LANE_WAVES); by default the whole sequence
@@ -1911,6 +1918,17 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
       const u64 share = sm.share;
       if (lane == 0) first = sm.base + atomicAdd((unsigned long long*)ticket, (unsigned long long)share);
       first = __shfl_sync(kAll, first, 0);  // every lane has read sm.share
+      // Mixed batches: one warp of a block looks for frequent keys, the others
+      // while a sixteenth of the ops looked at were settled so.  Batches that
+      // add to such keys gain much (16.8M Zipf(0.99) ops on a 2^27-slot table,
+      // the hottest keys among the added ones: DoubleHT 7.3 -> 17.0 Gops/s,
+      // DoubleHT(M) 10.8 -> 17.9, P2HT(M) 10.0 -> 13.3), looking costs the others
+      // 2-7%, and not looking 1-2%.
+      if (KIND == KIND_MIXED && hot && lane == 0) {
+        if (sm.hot_on) atomicAdd(&hot->looked, (u32)share);
+        const u32 hits = *reinterpret_cast<volatile u32*>(&hot->hits);
+        sm.hot_on = (threadIdx.x < 32) || (hits && hits * 16u >= *reinterpret_cast<volatile u32*>(&hot->looked));
+      }
       if (first < a.n) {
         next = first;
         end = (a.n - first < share) ? a.n : first + share;
@@ -1928,6 +1946,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         exhausted = true;
       }
     }
+    // upserts always look for frequent keys; mixed batches as above
+    const bool look = kHot && hot && (KIND == KIND_UPSERT || sm.hot_on);
     if (empty && next < end && __popc(parked) < NT) {
       const u64 rank = (u64)__popc(empty & ((1u << lane) - 1u));
       if (ring) {  // the ring's copies (usually complete long ago) become visible to the warp
@@ -1966,8 +1986,9 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
                 : SCHEME == SCHEME_DOUBLE            ? Ops::LW_INSERT_FREE
                 : front                              ? Ops::LW_INSERT_FRONT
                                                      : Ops::LW_UPDATE_ONLY;
-          if (kHot && hot && hot->settle(h1, K, V, op, twice)) {
+          if (kHot && look && (KIND == KIND_UPSERT || code == MX_ADD) && hot->settle(h1, K, V, op, twice)) {
             settled = true;
+            if (KIND == KIND_MIXED) atomicAdd(&hot->hits, 1u);
             if (a.vals_out) a.vals_out[gi] = 0;
             if (a.status_out) a.status_out[gi] = ST_FOUND;
           }
@@ -1975,7 +1996,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         if (!settled) {
           sm.key[lane] = K;
           sm.val[lane] = V;
-          sm.op[lane] = kHot ? (u8)twice : code;
+          sm.op[lane] = KIND == KIND_MIXED ? code : 0;
+          if (kHot && look && twice) sm.op[lane] = code | kTwice;
           sm.h1[lane] = h1;
           sm.h2[lane] = h2;
           sm.out[lane] = gi;  // the op's index
@@ -2014,7 +2036,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
       }
       next += ncons;
       // lanes whose ops were settled by HotKeys take more before the wave
-      if (kHot && hot && !ring && next < end && __popc(__ballot_sync(kAll, state == L_EMPTY)) >= 4) continue;
+      if (kHot && look && !ring && next < end && __popc(__ballot_sync(kAll, state == L_EMPTY)) >= 4) continue;
     }
     // 2. one wave: copy each active lane's current bucket, then settle
     const unsigned act = __ballot_sync(kAll, state == L_ACTIVE);
@@ -2057,7 +2079,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
                              KIND != KIND_ERASE);
         const bool wrote = r > 0 && st == ST_INSERTED;
         if (r > 0) {
-          if (kHot && hot && sm.op[lane] && st <= ST_INSERTED) hot->admit(sm.h1[lane], sm.key[lane], out);
+          if (kHot && look && (sm.op[lane] & kTwice) && st <= ST_INSERTED) hot->admit(sm.h1[lane], sm.key[lane], out);
           if (opk != Ops::LW_QUERY && opk != Ops::LW_ERASE) out = 0;
           const u64 gi = sm.out[lane];
           if (a.vals_out) a.vals_out[gi] = out;
@@ -2120,7 +2142,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         } else if (KIND == KIND_ERASE) {
           sj = Ops::template do_erase<false>(tv, c, Kj, h1j, h2j, no_pre(), o, rd);  // an erase-only launch
         } else {
-          sj = Ops::do_mixed(tv, c, sm.op[j], Kj, h1j, h2j, sm.val[j], no_pre(), o, rd);
+          sj = Ops::do_mixed(tv, c, sm.op[j] & (kTwice - 1), Kj, h1j, h2j, sm.val[j], no_pre(), o, rd);
         }
         if (c.tl == 0) {
           if (a.vals_out) a.vals_out[gj] = o;
@@ -2151,7 +2173,7 @@ constexpr u64 kStreamShare = 256;  // ops a streaming warp takes per ticket
 enum { PATH_EITHER = 0, PATH_STREAM = 1, PATH_CHUNK = 2 };
 template <int SCHEME, bool META, int B, int T, int KIND, bool INS, int PATH>
 __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchArgs a) {
-  constexpr bool kHot = KIND == KIND_UPSERT && !INS && PATH == PATH_STREAM;
+  constexpr bool kHot = (KIND == KIND_UPSERT || KIND == KIND_MIXED) && !INS && PATH == PATH_STREAM;
   __shared__ WarpSmem s_w[kWarps];
   __shared__ long long s_cnt;
   __shared__ HotKeys s_hot;
@@ -2240,6 +2262,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     const u64 end = a.n - begin < first ? a.n : begin + first;
     s_w[w].base = base;  // the same value on every lane
     s_w[w].share = share;
+    s_w[w].hot_on = w == 0;
     __syncwarp();
     dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, begin, end, s_w[w], lane, ticket, hot,
                                                     front);
@@ -2249,7 +2272,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     if (lane == 0 && mine) atomicAdd((unsigned long long*)&s_cnt, (unsigned long long)(long long)mine);
   }
   __syncthreads();  // every warp of the block is done with the ticket
-  if (kHot) hot->flush(tv, op);
+  if (kHot) hot->flush(tv, KIND == KIND_MIXED ? (int)OP_ADD : op);
   if (threadIdx.x == 0) {
     if ((KIND != KIND_QUERY && KIND != KIND_PROBE) && s_cnt)
       atomicAdd((unsigned long long*)&tv.ctr->count, (unsigned long long)s_cnt);

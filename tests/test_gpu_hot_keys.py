@@ -66,3 +66,39 @@ def test_frequent_keys(oracle_mod, scheme, meta, n_keys, op):
         np.add.at(want, pick, vals)
         assert (host(t.query(dev(uniq))) == want).all()
     t.close()
+
+
+@pytest.mark.parametrize("n_keys", [12, 400])
+@pytest.mark.parametrize("scheme,meta", DESIGNS, ids=DESIGN_IDS)
+def test_frequent_keys_in_mixed_batches(oracle_mod, scheme, meta, n_keys):
+    """Every code on its own skewed keys, the added ones above all: sums,
+    maxima, queried values and the counts of each status are the oracle's."""
+    import paper_2509_16407_gb300 as ws
+    n = 400003
+    t = ws.Table(1 << 14, scheme, meta)
+    om = oracle_mod.OracleMap()
+    uniq = W.distinct_keys(800 + n_keys, 6 * n_keys)
+    old = uniq[::2]
+    t.insert(dev(old), dev(old))
+    om.insert(old, old)
+    code = np.where(W.splitmix64(801, n) % np.uint64(3) == 0, W.splitmix64(802, n) % np.uint64(6), W.MX_ADD).astype(np.uint8)
+    keys = uniq.reshape(6, n_keys)[code, W.zipf(803, n, n_keys, 1.05) - 1]  # a key has one code
+    vals = W.splitmix64(804, n) >> np.uint64(8)
+    one = (code == W.MX_REPLACE) | (code == W.MX_INSERT)
+    vals[one] = W.mix13(keys[one])  # which copy wins does not show
+    v, st = t.mixed(dev(code), dev(keys), dev(vals))
+    wv, wst = om.mixed(code, keys, vals)
+    v, st = host(v), host(st)
+    for c in range(6):
+        m = code == c
+        assert (np.bincount(st[m], minlength=6) == np.bincount(wst[m], minlength=6)).all()
+        if c == W.MX_QUERY:
+            assert (v[m] == wv[m]).all()
+        elif c != W.MX_ERASE:
+            assert (v[m] == 0).all()
+    got, gst = t.query(dev(uniq), return_status=True)
+    want, ost = om.query(uniq)
+    assert (host(got) == want).all() and (host(gst) == ost).all()
+    assert t.count() == om.count()
+    check_layout(oracle_mod, t, om.count())
+    t.close()
