@@ -337,12 +337,16 @@ ws_status wsi::table_create(const ws_config* cfg, cudaStream_t stream, ws_table*
   std::memset(&tv, 0, sizeof(tv));
   // One lock bit per four slots (eight per 32-slot bucket), so that the ops in
   // flight rarely meet on one; at least 2^16 bits, which spreads a small
-  // table's lock atomics over 64 lines; and at most 2^22 (512 KiB): more would
-  // not stay in L2 beside a large table's traffic (one bit per four slots of a
-  // 2^27-slot table, 4 MiB, made its mixed batches 4% slower than 512 KiB),
-  // while 155k lanes on 2^22 bits miss 4% of their first attempts at most.
+  // table's lock atomics over 64 lines; and at most 2^23 (1 MiB; 2^22 under
+  // double hashing, where only mixed batches lock): more would not stay in L2
+  // beside a large table's traffic.  A mixed batch on a 2^27-slot DoubleHT(M)
+  // is 4% slower with 4 MiB than with 512 KiB; 13.4M inserts into a 2^28-slot
+  // P2HT, where 155k lanes in flight miss 4% of their first attempts on 2^22
+  // bits, take 2578 us with those, 2529 with 2^23 and 2517 with 2^24, which
+  // costs mixed batches on 2^27 slots up to 2%.
+  const u64 most = 1ull << (cfg->scheme == WS_DOUBLE ? 22 : 23);
   u64 lock_bits = t->S / 4;
-  lock_bits = lock_bits < (1ull << 16) ? (1ull << 16) : lock_bits > (1ull << 22) ? (1ull << 22) : lock_bits;
+  lock_bits = lock_bits < (1ull << 16) ? (1ull << 16) : lock_bits > most ? most : lock_bits;
   tv.lock_shift = 64;
   while ((1ull << (64 - tv.lock_shift)) < lock_bits) --tv.lock_shift;
   t->lock_words = lock_bits / 32;

@@ -2317,14 +2317,18 @@ cudaError_t launch_sized(const TableView& tv, const BatchArgs& a, cudaStream_t s
 // buckets, which rounds fetch in fewer dependent steps than streaming lanes
 // reading a line per wave (measured at 2^28 slots: negative queries 2.56 ms in
 // rounds vs 3.54 by lines, positive queries 1.51 vs 1.31, upserts 1.87 vs
-// 1.66); WS_OPT_STREAM = 2 streams them too.
+// 1.66); WS_OPT_STREAM = 2 streams them too.  Insert-if-unique calls on locking
+// tables that were ever erased always lock first, in chunks: the kernel for
+// either path would only spill more.
 template <int SCHEME, bool META, int B, int T, int KIND, bool INS = false>
 cudaError_t launch_path(const TableView& tv, const BatchArgs& a, cudaStream_t s, int num_sms) {
   constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
   constexpr int kStream = INS && SCHEME != SCHEME_DOUBLE ? PATH_EITHER : PATH_STREAM;
   const bool rounds = kRounds && (KIND == KIND_QUERY || KIND == KIND_ERASE) && tv.stream != 2;
-  return !tv.stream || rounds ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, PATH_CHUNK>>(tv, a, s, num_sms)
-                              : launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, kStream>>(tv, a, s, num_sms);
+  const bool locks = kStream == PATH_EITHER && !tv.shortcut;
+  return !tv.stream || rounds || locks
+             ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, PATH_CHUNK>>(tv, a, s, num_sms)
+             : launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, kStream>>(tv, a, s, num_sms);
 }
 
 template <int SCHEME, bool META, int B, int T>
