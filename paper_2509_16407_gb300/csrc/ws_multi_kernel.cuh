@@ -101,7 +101,16 @@ __global__ void __launch_bounds__(kThreads, 4) multi_kernel(MultiGroup g) {
       int d = multi_share<SCHEME, META, B, T, KIND>(it, begin, begin + n_here, s_w[w], lane);
       if (KIND != KIND_QUERY) {
         d = __reduce_add_sync(0xffffffffu, d);
-        if (lane == 0 && d) atomicAdd((unsigned long long*)&it.tv.ctr->count, (unsigned long long)(long long)d);
+        if (lane == 0 && d) {
+          const unsigned long long was =
+              atomicAdd((unsigned long long*)&it.tv.ctr->count, (unsigned long long)(long long)d);
+          // Two-choice and iceberg tables: the next single-table insert reads
+          // its load from `live` as long as nothing was erased, and until then
+          // `count` only grows.  Left behind, a table filled here looks empty
+          // to it: keys then go in without their locks at loads where that
+          // is slower and less even.
+          if (SCHEME != SCHEME_DOUBLE && d > 0) atomicMax((unsigned long long*)&it.tv.ctr->live, was + d);
+        }
       }
       __syncwarp();  // the share's results are written
       if (KIND == KIND_MIXED && g.host) {

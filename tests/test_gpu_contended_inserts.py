@@ -94,3 +94,28 @@ def test_fill_across_the_lock_line(ws, oracle_mod, scheme, meta, B, log2, slices
         assert oracle_mod.candidates_full(L["slots"], L["tags"], L["nb"], L["B"], L["scheme"], L["pmax"], L["seed1"],
                                           L["seed2"], failed).all()
     t.close()
+
+
+@pytest.mark.parametrize("meta", [False, True], ids=["P2HT", "P2HT(M)"])
+@pytest.mark.parametrize("kind", ["insert", "add"])
+def test_batched_fill_counts_as_load(ws, meta, kind):
+    """A two-choice table that a batch plan has filled to 0.7 is no low-load
+    table to the next single-table insert: every key takes its lock (shown by
+    locks that are all taken), as in a table filled by single-table calls."""
+    S = 1 << 14
+    t = ws.Table(S, "p2", meta, tile=8, spin_limit=64)
+    n = int(0.7 * S)
+    keys = W.distinct_keys(4600, n + 1000)
+    kd, st = dev(keys[:n]), dev(np.zeros(n, np.uint8))
+    item = (t, ws.BK_INSERT if kind == "insert" else ws.BK_UPSERT, kd, kd, None, st, 0)
+    plan = ws.BatchPlan([item + (("add",) if kind == "add" else ())])
+    assert plan.info()["fallback_items"] == 0
+    plan.launch()
+    assert (host(st) == ws.INSERTED).all() and t.count() == n
+    t.debug_fill_locks(True)
+    new = dev(keys[n:])
+    assert (host(t.insert(new, new, return_status=True)) == ws.FAIL_TIMEOUT).all()
+    t.debug_fill_locks(False)
+    assert (host(t.insert(new, new, return_status=True)) == ws.INSERTED).all()
+    plan.close()
+    t.close()
