@@ -15,7 +15,10 @@ cudaError_t launch_multi_7(int kind, const MultiGroup& g, cudaStream_t s, int nu
 namespace {
 __global__ void counts_kernel(const MultiItem* items, u32 n, u64* counts) {
   const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) counts[i] = items[i].tv.ctr->count;
+  if (i >= n) return;
+  const u64 c = items[i].tv.ctr->count;
+  items[i].tv.ctr->live = c;  // items outside the menu ran as single-table mixed kernels, which do not note it
+  counts[i] = c;
 }
 }  // namespace
 

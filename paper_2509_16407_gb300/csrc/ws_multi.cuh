@@ -87,7 +87,8 @@ inline int multi_menu_index(int scheme, bool meta, int B, int T) {
 cudaError_t launch_multi(int cfg, int kind, const MultiGroup& g, cudaStream_t s, int num_sms);
 
 // counts[i] = live keys of item i's table (counts: the device's view of
-// page-locked host memory), after the launches before it on the stream.
+// page-locked host memory), after the launches before it on the stream; the
+// tables note it as their load.
 cudaError_t launch_counts(const MultiItem* items, u32 n, u64* counts, cudaStream_t s);
 
 }  // namespace ws

@@ -119,3 +119,27 @@ def test_batched_fill_counts_as_load(ws, meta, kind):
     assert (host(t.insert(new, new, return_status=True)) == ws.INSERTED).all()
     plan.close()
     t.close()
+
+
+@pytest.mark.parametrize("scheme,plain", [("iceberg", False), ("p2", True)])
+def test_served_fill_counts_as_load(ws, scheme, plain):
+    """The same for a table that a server's requests have filled to 0.8 by
+    single-table kernels (no menu entry, or one launch per request)."""
+    import ctypes
+    S = 1 << 14
+    sv = ws.Server(grow_at=0, plain=plain)
+    tid = sv.add_table(S, scheme, True)
+    n = int(0.8 * S)
+    keys = W.distinct_keys(4700, n + 500)
+    sv.submit(tid, np.full(n, ws.MX_INSERT, np.uint8), keys[:n], keys[:n])
+    done = sv.drain()
+    assert len(done) == 1 and (done[0]["st"] == ws.INSERTED).all()
+    h, L = sv.table_handle(tid), ws.lib()
+    st = np.zeros(500, np.uint8)
+    new = np.ascontiguousarray(keys[n:])
+    for locked, want in ((1, ws.FAIL_TIMEOUT), (0, ws.INSERTED)):
+        assert L.ws_set_spin_limit(h, 64 if locked else 65536) == 0 and L.ws_debug_fill_locks(h, locked, None) == 0
+        assert L.ws_insert_ex(h, new.ctypes.data, new.ctypes.data, 500, st.ctypes.data, None) in (0, 5)
+        assert sv.count(tid) == n + (0 if locked else 500)  # waits for the call
+        assert (st == want).all()
+    sv.close()
