@@ -341,7 +341,8 @@ ws_status ws_batch_run_noalloc(const ws_batch_item* items, uint64_t n_items, ws_
 /* ---------------------------------------------------------------------------
  * Serving: a continuous-batching request loop over device-resident tables.
  * A request is a mixed op batch (ws_mixed_op codes) on one table, with HOST
- * buffers (pinned recommended) that must stay valid until its completion is
+ * buffers (pinned, with 8-byte aligned u64 arrays, recommended: only those are
+ * read and written in place) that must stay valid until its completion is
  * polled.  A worker thread keeps up to max_inflight launches on the GPU; each
  * launch runs the waiting requests of distinct tables (per-table FIFO, oldest
  * first, at most one request per table in flight) in one persistent
@@ -386,6 +387,10 @@ ws_status ws_server_add_table(ws_server* s, uint64_t capacity, ws_scheme scheme,
                               uint32_t* id);
 /* Thread-safe; returns at once.  n <= max_batch_ops. */
 ws_status ws_server_submit(ws_server* s, const ws_request* r, uint64_t* id);
+/* 1 when a launch would read and write the request's buffers in place (all of
+ * them page-locked and mapped, u64 arrays 8-byte aligned, results apart from
+ * the inputs), 0 when it would copy them.  Launches nothing. */
+int ws_debug_request_in_place(const ws_request* r);
 /* Up to max completions (waits up to wait_ms for the first). */
 ws_status ws_server_poll(ws_server* s, ws_completion* out, uint64_t max, uint64_t* n_out, int wait_ms);
 /* Stop (paused != 0) or resume admitting requests into new launches; work

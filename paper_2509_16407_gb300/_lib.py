@@ -91,6 +91,7 @@ SIGNATURES = {
     "ws_server_create": (st, [ctypes.POINTER(WsServerConfig), ctypes.POINTER(vp)]),
     "ws_server_add_table": (st, [vp, u64, i32, i32, i32, ctypes.POINTER(ctypes.c_uint32)]),
     "ws_server_submit": (st, [vp, ctypes.POINTER(WsRequest), ctypes.POINTER(ctypes.c_uint64)]),
+    "ws_debug_request_in_place": (i32, [ctypes.POINTER(WsRequest)]),
     "ws_server_poll": (st, [vp, ctypes.POINTER(WsCompletion), u64, ctypes.POINTER(ctypes.c_uint64), i32]),
     "ws_server_drain": (st, [vp]),
     "ws_server_pause": (st, [vp, i32]),

@@ -141,8 +141,6 @@ void* wsi::mapped_host(const void* p) {
 
 namespace {
 
-bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
-
 // WS_OPT_HOST_DIRECT: replace a host pointer by the device's view of it when
 // the memory is page-locked and mapped, so the kernel reads (and writes) it
 // in place over the host link instead of through the staging copies.

@@ -80,6 +80,7 @@ cudaError_t dispatch(const ws_table* t, const ws::TableView& tv, const ws::Batch
 // 1 device pointer on `device`, 2 host, 3 another device, 0 null.
 int classify(const void* p, int device);
 enum { PTR_NULL = 0, PTR_DEVICE = 1, PTR_HOST = 2, PTR_OTHER_DEVICE = 3 };
+inline bool aligned8(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
 // The device's view of page-locked, mapped host memory, or null (pageable
 // memory, or a pointer that is not host memory).
 void* mapped_host(const void* p);

@@ -342,11 +342,14 @@ void wake_worker(ws_server* sv) {
 }
 
 // Device views of a request's buffers, or keys == nullptr when one of them is
-// not page-locked and mapped, or results overlap inputs other than their own.
+// not page-locked and mapped, a u64 array is not 8-byte aligned (the kernel
+// moves whole elements; the copy engines take any address, so such a request is
+// served all the same), or results overlap inputs other than their own.
 ws::HostOps host_ops(const ws_request& r) {
   ws::HostOps h = {};
   const u64 n = r.n;
-  if (n == 0 || crosses(r.vals_out, 8, r.keys, 8, n) || crosses(r.vals_out, 8, r.vals, 8, n) ||
+  if (n == 0 || !aligned8(r.keys) || !aligned8(r.vals) || !aligned8(r.vals_out)) return h;
+  if (crosses(r.vals_out, 8, r.keys, 8, n) || crosses(r.vals_out, 8, r.vals, 8, n) ||
       crosses(r.vals_out, 8, r.ops, 1, n) || crosses(r.status_out, 1, r.keys, 8, n) ||
       crosses(r.status_out, 1, r.vals, 8, n) || crosses(r.status_out, 1, r.ops, 1, n) ||
       crosses(r.status_out, 1, r.vals_out, 8, n))
@@ -515,6 +518,10 @@ ws_status ws_server_submit(ws_server* sv, const ws_request* r, uint64_t* id) {
   sv->cv_in.notify_one();
   if (id) *id = q.id;
   return WS_OK;
+}
+
+int ws_debug_request_in_place(const ws_request* r) {
+  return r && (!r->n || (r->ops && r->keys)) && host_ops(*r).keys ? 1 : 0;
 }
 
 ws_status ws_server_poll(ws_server* sv, ws_completion* out, uint64_t max, uint64_t* n_out, int wait_ms) {
