@@ -13,6 +13,12 @@ cudaError_t launch_multi_6(int kind, const MultiGroup& g, cudaStream_t s, int nu
 cudaError_t launch_multi_7(int kind, const MultiGroup& g, cudaStream_t s, int num_sms);
 
 namespace {
+__global__ void count_kernel(Counters* ctr, u64* count) {
+  const u64 c = ctr->count;
+  ctr->live = c;  // as below
+  *count = c;
+}
+
 __global__ void counts_kernel(const MultiItem* items, u32 n, u64* counts) {
   const u32 i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -25,6 +31,11 @@ __global__ void counts_kernel(const MultiItem* items, u32 n, u64* counts) {
 cudaError_t launch_counts(const MultiItem* items, u32 n, u64* counts, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   counts_kernel<<<(n + 127) / 128, 128, 0, s>>>(items, n, counts);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_count(const TableView& tv, u64* count, cudaStream_t s) {
+  count_kernel<<<1, 1, 0, s>>>(tv.ctr, count);
   return cudaGetLastError();
 }
 

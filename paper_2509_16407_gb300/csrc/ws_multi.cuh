@@ -90,5 +90,7 @@ cudaError_t launch_multi(int cfg, int kind, const MultiGroup& g, cudaStream_t s,
 // page-locked host memory), after the launches before it on the stream; the
 // tables note it as their load.
 cudaError_t launch_counts(const MultiItem* items, u32 n, u64* counts, cudaStream_t s);
+// The same for one table whose descriptor the host has.
+cudaError_t launch_count(const TableView& tv, u64* count, cudaStream_t s);
 
 }  // namespace ws

@@ -267,10 +267,10 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     }
   }
   group_off[ws::kMultiMenu] = nchunks;
-  if (ok)
-    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * kItemBytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
   if (ok && nchunks) {
-    ok = cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
+    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * kItemBytes, cudaMemcpyHostToDevice, s) ==
+             cudaSuccess &&
+         cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
              cudaSuccess &&
          cudaMemsetAsync(sl.d_ticket, 0, ws::kMultiMenu * sizeof(u32), s) == cudaSuccess;
     for (int cfg = 0; cfg < ws::kMultiMenu && ok; ++cfg) {
@@ -297,7 +297,11 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     sv->tables[sl.tabs[i]].t->last_stream = s;
     off += n;
   }
-  if (ok) ok = ws::launch_counts(sl.d_items, (u32)sl.reqs.size(), sl.m_counts, s) == cudaSuccess;
+  // Without a multi-table kernel (plain mode) no descriptors were sent: sending
+  // them for the counts alone took 4 us of a plain request's 97 (200 ops).
+  if (ok && nchunks) ok = ws::launch_counts(sl.d_items, (u32)sl.reqs.size(), sl.m_counts, s) == cudaSuccess;
+  for (size_t i = 0; i < sl.reqs.size() && ok && !nchunks; ++i)
+    ok = ws::launch_count(sl.h_items[i].tv, sl.m_counts + i, s) == cudaSuccess;
   if (ok) ok = cudaEventRecord(sl.done, s) == cudaSuccess;
   if (!ok) {
     note_cuda(cudaGetLastError(), "server launch");
@@ -354,12 +358,13 @@ ws::HostOps host_ops(const ws_request& r) {
       crosses(r.status_out, 1, r.vals, 8, n) || crosses(r.status_out, 1, r.ops, 1, n) ||
       crosses(r.status_out, 1, r.vals_out, 8, n))
     return h;
+  const u64* keys = static_cast<const u64*>(mapped_host(r.keys));
+  if (!keys) return h;  // pageable requests: one look at a pointer
   h.vals = static_cast<const u64*>(mapped_host(r.vals));
   h.ops = static_cast<const u8*>(mapped_host(r.ops));
   h.vals_out = static_cast<u64*>(mapped_host(r.vals_out));
   h.status_out = static_cast<u8*>(mapped_host(r.status_out));
-  if (h.ops && (h.vals || !r.vals) && (h.vals_out || !r.vals_out) && (h.status_out || !r.status_out))
-    h.keys = static_cast<const u64*>(mapped_host(r.keys));
+  if (h.ops && (h.vals || !r.vals) && (h.vals_out || !r.vals_out) && (h.status_out || !r.status_out)) h.keys = keys;
   return h;
 }
 
