@@ -184,9 +184,9 @@ ws_status ws_set_spin_limit(ws_table* t, uint32_t spins);
  *  chunks (copy engines, eight chunk buffers rotating against the kernels).
  *  1: the kernels read keys, values and op codes in place over the host
  *  link; host result buffers are still staged, except by calls of at most 2^19
- *  ops, which write them in place.  2: results are always written in place
- *  too.  3: 1 for insert-if-unique and erase calls (their probe
- *  sequences hide the host link's latency), 0 for queries, upserts and mixed
+ *  ops (mixed calls that return values: 2^18), which write them in place.  2:
+ *  results are always written in place too.  3: 1 for insert-if-unique and
+ *  erase calls (their probe sequences hide the host link's latency), 0 for queries, upserts and mixed
  *  batches (whose kernels are short per op and read inputs faster from
  *  device memory).  Pageable host memory is always staged.  The caller must
  *  not touch the buffers until the call's work on its stream has completed.

@@ -212,15 +212,21 @@ ws_status run_batch(ws_table* t, int kind, int op, const u8* ops, const uint64_t
   const u32 in_flags = host_in ? (u32)ws::BATCH_HOST_INPUTS : 0u;
   // Results written in place: by small calls too, whose staging (two copies
   // and four events) costs more than the scattered writes over the host link.
-  // Lookups with page-locked keys and results, back to back, in place against
-  // staged: 100,000 18 us against 31, 400,000 53 against 58, 1M 118 against
-  // 115, 3M 347 against 292.
-  constexpr u64 kSmallDirect = 1ull << 19;
+  // Back to back on a 2^26-slot table, all buffers page-locked, in place
+  // against staged, DoubleHT / P2HT(M), us per call of 2^18 and of 2^19 ops:
+  // lookups (values and status) 25 / 27 against 50 / 52 and 43 / 47 against
+  // 80 / 87, inserts 40 / 50 against 51 / 66 and 64 / 78 against 74 / 97, upserts
+  // 32 / 33 against 40 / 45 and 52 / 54 against 62 / 67, erases 36 / 35 against
+  // 49 / 53 and 65 / 65 against 74 / 89, mixed (values and status) 54 / 55
+  // against 59 / 61 and 98 / 99 against 92 / 97.  A mixed call has the most bytes
+  // on the link in both directions; with a status alone it gains at 2^19 too (59
+  // against 66).  Lookups of 1M: 118 against 115, 3M: 347 against 292.
+  const u64 small_direct = kind == ws::KIND_MIXED && vals_out ? 1ull << 18 : 1ull << 19;
   const bool apart = !crosses(vals_out, 8, keys0, 8, n) && !crosses(vals_out, 8, vals0, 8, n) &&
                      !crosses(vals_out, 8, ops0, 1, n) && !crosses(status_out, 1, keys0, 8, n) &&
                      !crosses(status_out, 1, vals0, 8, n) && !crosses(status_out, 1, ops0, 1, n) &&
                      !crosses(status_out, 1, vals_out, 8, n);
-  if (hd >= 2 || (hd == 1 && n <= kSmallDirect && apart)) {
+  if (hd >= 2 || (hd == 1 && n <= small_direct && apart)) {
     go_direct(vals_out, pvo);
     go_direct(status_out, pst);
   }
