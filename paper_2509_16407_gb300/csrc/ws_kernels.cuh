@@ -1561,7 +1561,11 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   }
   int snap_wave = -1;
 
-  constexpr int kPasses = (KIND == KIND_UPSERT || KIND == KIND_MIXED) ? kChunkPasses : 1;
+  // Lanes that take no lock (plain two-choice buckets wider than their snapshot,
+  // other than by rounds) never go round again; the loop alone took a quarter
+  // more (4M present keys inserted into a 2^26-slot P2HT of 16-slot buckets:
+  // 548 us with it, 421 without).
+  constexpr int kPasses = ((KIND == KIND_UPSERT || KIND == KIND_MIXED) && kLaneLock) ? kChunkPasses : 1;
   bool again = false;  // run the op through the lane path once more
   if (kRounds) {
     // Whole-bucket rounds: eight buckets per round, one op's bucket per copy
