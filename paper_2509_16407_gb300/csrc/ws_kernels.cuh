@@ -805,8 +805,8 @@ struct TileOps {
   // keys build a 2^16-slot DoubleHT, 5 are in flight per bucket, and the build
   // took 60 us with a new probe after each lost claim, 22 us with this.  (With
   // more lock bits and lane passes, 6.7M inserts into a 2^23-slot IcebergHT(M)
-  // went from 1387 to 650 us, 209,715 into a 2^22-slot P2HT(M) from 145 to
-  // 62 us.)  Returns 1 claimed, 2 the slot at idx holds K (plain tables), 0
+  // went from 1387 to 650 us.)  Two-choice claims stay where they are (see
+  // claim_limit).  Returns 1 claimed, 2 the slot at idx holds K (plain tables), 0
   // lost.
   __device__ static __forceinline__ int lane_claim(const TableView& tv, u64& idx, u64 limit, u64 fk, u64 fv, u64 K,
                                                    u64 V) {
@@ -830,15 +830,30 @@ struct TileOps {
     }
   }
   // How far a claim may move on from slot idx.  Where the scheme leaves no
-  // choice, to the end of the bucket (two choices: to the 3/4 threshold).
-  // Between two buckets, while the chosen one -- `spare` slots emptier than
-  // the other when they were read, and one fuller with every lost claim -- is
-  // not the fuller one: going on to the end of the bucket left iceberg tables
-  // of 2^12 to 2^17 slots with 3 to 13 FULL keys at 0.95, where there were
-  // none.
+  // choice, to the end of the bucket.  Between two backyard buckets, while the
+  // chosen one -- `spare` slots emptier than the other when they were read, and
+  // one fuller with every lost claim -- is not the fuller one: going on to the
+  // end of the bucket left iceberg tables of 2^12 to 2^17 slots with 3 to 13
+  // FULL keys at 0.95, where there were none.  Two choices: not at all.  A key
+  // without a choice that moved on would get in ahead of the keys that have one
+  // and must read both their buckets again after a lost claim: buckets would
+  // fill to the threshold from the keys without a choice, which loses the
+  // evenness that two choices are for wherever several ops are in flight per
+  // bucket.  (The lane passes and restarts of two-choice inserts are limited for
+  // the same reason, see kTwoChoicePasses.)  Keys without a slot when a P2HT is
+  // filled to 0.95 by one insert / one upsert-add call, means of 24 tables (4 of
+  // 2^20), and us per call:
+  //   2^14 slots  moving on to the threshold, 8 passes  18 / 24    106 / 180
+  //               so                                     3 / 3     421 / 385
+  //   2^17 slots  moving on                             52 / 61    174 / 428
+  //               so                                    22 / 23   1412 / 1270
+  //   2^20 slots  moving on                            235 / 295   298 / 877
+  //               so                                   190 / 216   827 / 1698
+  // (one key after another: 2.3, 18 and 144).  From 2^22 slots on the counts are
+  // equal and so takes 1-7% longer (2^22 slots, P2HT(M) 455 -> 514 us).
   __device__ static __forceinline__ u64 claim_limit(u64 idx, bool choice, u32 spare) {
-    const u64 first = idx & ~(u64)(B - 1);
-    const u64 end = first + (SCHEME == SCHEME_P2 && !choice ? (u64)FILL_SHORTCUT : (u64)B);
+    if (SCHEME == SCHEME_P2) return idx + 1;
+    const u64 end = (idx & ~(u64)(B - 1)) + (u64)B;
     return !choice || idx + 1 + spare > end ? end : idx + 1 + spare;
   }
 
@@ -1203,8 +1218,8 @@ struct TileOps {
       return 1;
     }
     u64 idx = ch == 0 ? ls.ff_idx : ls.f1_idx;
-    const bool choice = ls.occ0 >= FILL_SHORTCUT;
-    if (lane_claim(tv, idx, claim_limit(idx, choice, 0), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) != 1) {
+    if (lane_claim(tv, idx, claim_limit(idx, false, 0), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) !=
+        1) {
       fresh = false;
       return -1;
     }
@@ -1332,8 +1347,6 @@ struct TileOps {
         st = ST_FULL;
         return 1;
       }
-      choice = ls.occ0 >= FILL_SHORTCUT;
-      if (w > 0) spare = ch == 1 ? (ls.occ0 > sn.occ ? ls.occ0 - sn.occ : 0) : (sn.occ > ls.occ0 ? sn.occ - ls.occ0 : 0);
       if (ch == (int)w) {  // the free slot of this wave's bucket
         if (META) {
           fidx = bw * 32 + (u64)sn.ffree;
@@ -1390,10 +1403,22 @@ __device__ __forceinline__ void count_failure(const TableView& tv, u8 st) {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 // 32-op chunks: lane passes of an insert whose lock or claim was lost before the
-// tiles take it (13,107 inserts into a 2^18-slot P2HT at 0.8 load: 138 us with 2
-// passes, 64 with 4, 57 with 8; large tables do not care).
+// tiles take it.  Streaming lanes: restarts of an op for the same reasons.
 constexpr int kChunkPasses = 8;
-constexpr int kLaneRestarts = 4;  // streaming lane: restarts of an op after a lost CAS before the tiles
+constexpr int kLaneRestarts = 4;
+// Two choices.  The tiles serialise the inserts of a bucket's keys, lanes that
+// try again at once favour the keys that read one bucket, so more passes fill a
+// small table less evenly (2^17-slot P2HT to 0.55 and then to 0.95: 37 keys
+// without a slot with 8 passes, 22 with 4; 8-slot buckets, 2^14 slots to 0.9: 292
+// with 8, 237 with 3, 225 with 2, in order 213) but faster (13,107 inserts into a
+// 2^18-slot P2HT at 0.8 load: 138 us with 2, 64 with 4, 57 with 8).  Large tables
+// do not care.  Restarts likewise: upsert-adds that fill a 2^20-slot P2HT to 0.95
+// leave 241 keys with 4 (1059 us), 233 with 3 (1350), 205 with 2 (1867); lanes of
+// metadata tables read a bucket in one wave and lose nothing with 4.
+template <int B>
+constexpr int kTwoChoicePasses = B == 32 ? 4 : 2;
+template <bool META>
+constexpr int kTwoChoiceRestarts = META ? kLaneRestarts : 2;
 
 struct WarpSmem {
   u64 key[32], val[32], out[32], h1[32], h2[32];
@@ -1551,7 +1576,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   // holders of that lock insert K).  Add / max / replace probe lock-free
   // first: a present key -- a hot Zipf key above all -- needs no lock.  An op
   // that proved its key absent without the lock tries for it before its next
-  // pass (kChunkPasses).
+  // pass (kPasses).
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || kRounds;
   const u64 b0 = Ops::bucket(tv, h1, h2, 0), lk = Ops::lock_of(tv, h2);
   bool locked = false;
@@ -1565,7 +1590,9 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   // other than by rounds) never go round again; the loop alone took a quarter
   // more (4M present keys inserted into a 2^26-slot P2HT of 16-slot buckets:
   // 548 us with it, 421 without).
-  constexpr int kPasses = ((KIND == KIND_UPSERT || KIND == KIND_MIXED) && kLaneLock) ? kChunkPasses : 1;
+  constexpr int kPasses = ((KIND == KIND_UPSERT || KIND == KIND_MIXED) && kLaneLock)
+                              ? (SCHEME == SCHEME_P2 ? kTwoChoicePasses<B> : kChunkPasses)
+                              : 1;
   bool again = false;  // run the op through the lane path once more
   if (kRounds) {
     // Whole-bucket rounds: eight buckets per round, one op's bucket per copy
@@ -1685,8 +1712,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
               done = true;
             } else {
               u64 idx = ch == 0 ? b0 * 32 + (u64)f0 : bc * 32 + (u64)fs;
-              const bool choice = occ0 >= Ops::FILL_SHORTCUT && c == 1;
-              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx, choice, 0), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K,
+              if (Ops::lane_claim(tv, idx, Ops::claim_limit(idx, false, 0), ch == 0 ? f0k : fk, ch == 0 ? f0v : fv, K,
                                   V) == 1) {
                 ++dcount;
                 st = ST_INSERTED;
@@ -1869,7 +1895,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 // cooperative tiles, which run only when no lane of the warp is active -- so
 // no lane of the warp holds a lock a tile might wait for.  An op that lost a
 // claim, or proved its key absent without the lock, first starts over in its
-// lane (kLaneRestarts).  Refill pauses once enough ops are parked to fill the tiles.
+// lane (kRestarts).  Refill pauses once enough ops are parked to fill the tiles.
 // -------------------------------------------------------------------------
 // Work shares: the warp serves [begin, end), and, unless `ticket` is null,
 // then takes shares of up to sm.share ops (a multiple of 32) of [sm.base, n)
@@ -1885,6 +1911,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
   constexpr int NT = 32 / T;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || Ops::kLines;
+  constexpr int kRestarts = SCHEME == SCHEME_P2 ? kTwoChoiceRestarts<META> : kLaneRestarts;
   constexpr bool kHot = KIND == KIND_UPSERT || KIND == KIND_MIXED;
   constexpr u8 kTwice = 0x80;  // in sm.op: the op's key is frequent
   const u64 ks = a.key_stride ? a.key_stride : 1;
@@ -2090,7 +2117,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           if (a.status_out) a.status_out[gi] = st;
           if (st >= ST_FULL) count_failure(tv, st);
           state = L_EMPTY;
-        } else if (((r == -2 && kLaneLock && !locked) || (r == -1 && !fresh)) && restarts < kLaneRestarts) {
+        } else if (((r == -2 && kLaneLock && !locked) || (r == -1 && !fresh)) && restarts < kRestarts) {
           // Absent without the lock: take it now, or -- its holder may be
           // inserting this very key -- look again without it.  Or a lost
           // claim: the table moved under the snapshot; a held lock stays held.
