@@ -139,9 +139,11 @@ class Table:
         if stream is None:
             torch = _torch()
             # a small query is host-bound (1000 keys: 18 us a call, of which 4
-            # went into the device check and a Stream object; 14 with the handle)
-            if torch.cuda.is_initialized():
-                return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(self.device))
+            # went into the device check and a Stream object; 14 with the handle,
+            # which torch has no public call for)
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            if raw is not None and torch.cuda.is_initialized():
+                return ctypes.c_void_p(raw(self.device))
             if torch.cuda.is_available():
                 return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
             return None
