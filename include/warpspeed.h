@@ -164,9 +164,15 @@ ws_status ws_set_spin_limit(ws_table* t, uint32_t spins);
  *  of the launch so the warps run dry together), a lane follows its op's probe
  *  sequence one bucket per wave and takes the next op as soon as its op
  *  settles; ops the lanes cannot settle go to the tiles.  0 serves 32-op
- *  chunks (lane waves, then tiles for what is left), as batched and serving
- *  launches always do, and as insert-if-unique calls on two-choice and
- *  iceberg tables do (their inserts lock: once per chunk beats once per wave).
+ *  chunks (lane waves, then tiles for what is left).  Insert-if-unique calls on
+ *  two-choice and iceberg tables lock before they probe, which chunks do once
+ *  per 32 ops, and use chunks too -- except into tables that were never erased
+ *  (a mixed call counts as an erase) and are not too full, by the live count
+ *  that the last call noted (iceberg below 3/4 of the slots halfway through the
+ *  call; two choices below 0.6 at its end, 0.45 for 8- and 16-slot buckets, and
+ *  plain ones below 1/2 halfway): those insert without the lock where the scheme
+ *  leaves no choice, in streaming lanes.  Batched and serving launches stream
+ *  256-op shares; their plain 32-slot two-choice tables use chunks.
  *  Queries and erases on two-choice tables with plain 32-slot buckets read
  *  whole buckets in 32-op chunks; 2 streams them too, reading a bucket line by
  *  line up to the key or the first EMPTY slot: fewer bytes for keys near the

@@ -129,6 +129,11 @@ int wsi::classify(const void* p, int device) {
   return PTR_HOST;
 }
 
+// The first byte decides for the whole array.  An array that runs past its
+// registered range is read in place all the same: beside a Grace host the
+// device reaches pageable memory through the host's page tables
+// (cudaDevAttrPageableMemoryAccessUsesHostPageTables is 1) at the same
+// addresses, while the copy engines refuse such a range (cudaErrorInvalidValue).
 void* wsi::mapped_host(const void* p) {
   if (!p) return nullptr;
   cudaPointerAttributes at;
@@ -281,7 +286,7 @@ ws_status run_batch(ws_table* t, int kind, int op, const u8* ops, const uint64_t
   return WS_OK;
 }
 
-// b_0 of each key (iceberg: the front-yard bucket, whose lock inserters take).
+// b_0 of each key (iceberg: the front-yard bucket).
 __global__ void primary_bucket_kernel(const u64* keys, u64* out, u64 n, u64 seed1, u64 mask, u64 nb_front,
                                       int iceberg) {
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {

@@ -890,12 +890,12 @@ struct TileOps {
   // LOCKFREE: the caller guarantees that no erase runs in the same launch (a
   // plain insert / upsert call is one phase).
   template <bool LOCKFREE>
-  // Writes read the table through L2 even in bulk-synchronous mode: the
-  // call's other inserts write the slots they probe, and a lost claim must
-  // see the winner (weak, L1-cacheable loads could return the stale line on
-  // every retry).  `tv` keeps the mode for the lock decisions.
   __device__ static u8 do_upsert(const TableView& tv_in, const TileCtx<T>& c, u64 K, u64 h1, u64 h2, u64 V, int op,
                                  PreRef pre, int& dcount) {
+    // Writes read the table through L2 even in bulk-synchronous mode: the
+    // call's other inserts write the slots they probe, and a lost claim must
+    // see the winner (weak, L1-cacheable loads could return the stale line on
+    // every retry).  `phased` keeps the mode for the lock decisions.
     TableView tv = tv_in;
     const bool phased = tv.phased != 0;
     tv.phased = 0;
@@ -932,8 +932,8 @@ struct TileOps {
       if (c.tl == 0) apply(tv, h.idx, op, V);
       return ST_FOUND;
     }
-    // Absent: take the primary bucket's lock so that inserters of this key
-    // agree on one slot (§4.1).  While another tile holds it -- often one
+    // Absent: take the key's lock so that inserters of this key agree on one
+    // slot (§4.1).  While another tile holds it -- often one
     // inserting this very key -- probe again lock-free: once the key is
     // present its slot never moves, so the update needs no lock.  This keeps
     // a batch's many copies of a hot key from queueing on one lock bit.
@@ -1411,7 +1411,7 @@ constexpr int kLaneRestarts = 4;
 // small table less evenly (2^17-slot P2HT to 0.55 and then to 0.95: 37 keys
 // without a slot with 8 passes, 22 with 4; 8-slot buckets, 2^14 slots to 0.9: 292
 // with 8, 237 with 3, 225 with 2, in order 213) but faster (13,107 inserts into a
-// 2^18-slot P2HT at 0.8 load: 138 us with 2, 64 with 4, 57 with 8).  Large tables
+// 2^18-slot P2HT at 0.8 load: 205 us with 2, 86 with 4, 78 with 8).  Large tables
 // do not care.  Restarts likewise: upsert-adds that fill a 2^20-slot P2HT to 0.95
 // leave 241 keys with 4 (1059 us), 233 with 3 (1350), 205 with 2 (1867); lanes of
 // metadata tables read a bucket in one wave and lose nothing with 4.
@@ -2226,10 +2226,10 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   // others did).  Speed, by the load halfway through the call: 0.75 for
   // iceberg, 0.5 for P2HT, whose streaming lanes read a bucket line by line.
   // 2^27 slots, a tenth of them inserted at 0.4-0.5 / 0.5-0.6 / 0.6-0.7 /
-  // 0.7-0.8 load, lock-free against lock first: IcebergHT(M) 1125 / 1164 / 1242
-  // / 1523 us against 1302 / 1329 / 1414 / 1460, P2HT(M) 1138 / 1169 / 1313 /
-  // 1667 against 1312 / 1324 / 1316 / 1332, P2HT 1188 / 1871 / 3574 / 5951
-  // against 1489 / 1604 / 1846 / 2261 (and 607 against 1452 into an empty
+  // 0.7-0.8 load, lock-free against lock first: IcebergHT(M) 1152 / 1198 / 1275
+  // / 1584 us against 1303 / 1335 / 1393 / 1433, P2HT(M) 1165 / 1194 / 1386 /
+  // 1789 against 1319 / 1329 / 1318 / 1334, P2HT 1200 / 1890 / 3599 / 5961
+  // against 1487 / 1587 / 1825 / 2238 (and 647 against 1451 into an empty
   // table).  Balance, by the load at the end of the call: keys without a choice
   // get in before keys in flight that have one, which costs two choices some of
   // their evenness.  Filling 2^22 slots to 0.95 with the first part in that

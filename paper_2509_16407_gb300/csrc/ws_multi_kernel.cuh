@@ -7,7 +7,9 @@ namespace ws {
 
 // One warp's share [begin, end) of a chunk of one item: streaming lanes, or
 // -- for two-choice tables with plain 32-slot buckets -- 32-op chunks with
-// whole-bucket rounds.  Returns the warp's count delta.
+// whole-bucket rounds.  Frequent keys (HotKeys) and inserts without the lock
+// (LW_INSERT_FRONT) are the single-table kernel's: copies of a Zipf-hot key in
+// one item queue on its line here.  Returns the warp's count delta.
 template <int SCHEME, bool META, int B, int T, int KIND>
 __device__ __forceinline__ int multi_share(const MultiItem& it, u64 begin, u64 end, WarpSmem& sm, int lane) {
   constexpr bool kRounds = (SCHEME == SCHEME_P2) && !META && B == 32;
