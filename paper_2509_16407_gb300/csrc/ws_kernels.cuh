@@ -849,7 +849,7 @@ struct TileOps {
   //               so                                    22 / 23   1412 / 1270
   //   2^20 slots  moving on                            235 / 295   298 / 877
   //               so                                   190 / 216   827 / 1698
-  // (one key after another: 2.3, 18 and 144).  From 2^22 slots on the counts are
+  // (one key after another: 2.8, 19 and 138).  From 2^22 slots on the counts are
   // equal and so takes 1-7% longer (2^22 slots, P2HT(M) 455 -> 514 us).
   __device__ static __forceinline__ u64 claim_limit(u64 idx, bool choice, u32 spare) {
     if (SCHEME == SCHEME_P2) return idx + 1;
