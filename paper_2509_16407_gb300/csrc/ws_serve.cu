@@ -267,10 +267,11 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     }
   }
   group_off[ws::kMultiMenu] = nchunks;
+  const bool sent = nchunks || sl.reqs.size() > 1;  // the launch's descriptors are on the device
+  if (ok && sent)
+    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * kItemBytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
   if (ok && nchunks) {
-    ok = cudaMemcpyAsync(sl.d_items, sl.h_items, sl.reqs.size() * kItemBytes, cudaMemcpyHostToDevice, s) ==
-             cudaSuccess &&
-         cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
+    ok = cudaMemcpyAsync(sl.d_chunks, sl.h_chunks, nchunks * sizeof(ws::MultiChunk), cudaMemcpyHostToDevice, s) ==
              cudaSuccess &&
          cudaMemsetAsync(sl.d_ticket, 0, ws::kMultiMenu * sizeof(u32), s) == cudaSuccess;
     for (int cfg = 0; cfg < ws::kMultiMenu && ok; ++cfg) {
@@ -297,11 +298,11 @@ bool launch_slot(ws_server* sv, Slot& sl) {
     sv->tables[sl.tabs[i]].t->last_stream = s;
     off += n;
   }
-  // Without a multi-table kernel (plain mode) no descriptors were sent: sending
-  // them for the counts alone took 4 us of a plain request's 97 (200 ops).
-  if (ok && nchunks) ok = ws::launch_counts(sl.d_items, (u32)sl.reqs.size(), sl.m_counts, s) == cudaSuccess;
-  for (size_t i = 0; i < sl.reqs.size() && ok && !nchunks; ++i)
-    ok = ws::launch_count(sl.h_items[i].tv, sl.m_counts + i, s) == cudaSuccess;
+  // A single request without a multi-table kernel (plain mode) needs no
+  // descriptor: sending it for the count alone took 4 us of 97 (200 ops).
+  if (ok)
+    ok = (sent ? ws::launch_counts(sl.d_items, (u32)sl.reqs.size(), sl.m_counts, s)
+               : ws::launch_count(sl.h_items[0].tv, sl.m_counts, s)) == cudaSuccess;
   if (ok) ok = cudaEventRecord(sl.done, s) == cudaSuccess;
   if (!ok) {
     note_cuda(cudaGetLastError(), "server launch");
