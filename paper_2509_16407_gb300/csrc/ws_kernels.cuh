@@ -1428,7 +1428,7 @@ struct WarpSmem {
     u8 list[32];                   // whole-bucket rounds: open ops of a bucket pass
     struct {                       // streaming lanes:
       u64 base, share;             // where ticketed shares start, ops of the next one
-      u32 hot_on;                  // mixed: the warp looks for frequent keys in this share
+      u32 hot_on;                  // the warp looks for frequent keys (mixed: in this share)
     };
   };
   u64 in_key[32], in_val[32];  // streaming lanes, host inputs: op i's key / value in slot i % 32
@@ -1977,8 +1977,7 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         exhausted = true;
       }
     }
-    // upserts always look for frequent keys; mixed batches as above
-    const bool look = kHot && hot && (KIND == KIND_UPSERT || sm.hot_on);
+    const bool look = kHot && hot && sm.hot_on;
     if (empty && next < end && __popc(parked) < NT) {
       const u64 rank = (u64)__popc(empty & ((1u << lane) - 1u));
       if (ring) {  // the ring's copies (usually complete long ago) become visible to the warp
@@ -2211,7 +2210,13 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   HotKeys* hot = kHot ? &s_hot : nullptr;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_cnt = 0;
-  if (kHot) hot->clear();
+  // Upserts and one warp of a mixed batch look for frequent keys, in launches of
+  // more than one op per lane (those that take tickets).  Smaller ones last less
+  // than the copies of a hot key take (DoubleHT upserts, us without looking and
+  // with: 300 ops 3.1 and 3.7; Zipf adds, 30,000 ops 9.2 and 10.2, 120,000 27.9 and
+  // 30.0, but 250,000 66 and 47).
+  const bool looks = kHot && a.n > 32ull * kWarps * gridDim.x;
+  if (looks) hot->clear();
   __syncthreads();
   const int op = INS ? (int)OP_INSERT : a.op;
   const bool lockfree = (KIND == KIND_UPSERT);  // one call is one phase: no erase runs with it
@@ -2293,7 +2298,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     const u64 end = a.n - begin < first ? a.n : begin + first;
     s_w[w].base = base;  // the same value on every lane
     s_w[w].share = share;
-    s_w[w].hot_on = w == 0;
+    s_w[w].hot_on = looks && (KIND == KIND_UPSERT || w == 0);
     __syncwarp();
     dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, begin, end, s_w[w], lane, ticket, hot,
                                                     front);
@@ -2303,7 +2308,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     if (lane == 0 && mine) atomicAdd((unsigned long long*)&s_cnt, (unsigned long long)(long long)mine);
   }
   __syncthreads();  // every warp of the block is done with the ticket
-  if (kHot) hot->flush(tv, KIND == KIND_MIXED ? (int)OP_ADD : op);
+  if (looks) hot->flush(tv, KIND == KIND_MIXED ? (int)OP_ADD : op);
   if (threadIdx.x == 0) {
     if ((KIND != KIND_QUERY && KIND != KIND_PROBE) && s_cnt)
       atomicAdd((unsigned long long*)&tv.ctr->count, (unsigned long long)s_cnt);
