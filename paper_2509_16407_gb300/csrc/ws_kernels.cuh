@@ -1428,7 +1428,7 @@ struct WarpSmem {
     u8 list[32];                   // whole-bucket rounds: open ops of a bucket pass
     struct {                       // streaming lanes:
       u64 base, share;             // where ticketed shares start, ops of the next one
-      u32 hot_on;                  // the warp looks for frequent keys (mixed: in this share)
+      u32 hot_on;                  // mixed: the warp looks for frequent keys in this share
     };
   };
   u64 in_key[32], in_val[32];  // streaming lanes, host inputs: op i's key / value in slot i % 32
@@ -1977,7 +1977,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
         exhausted = true;
       }
     }
-    const bool look = kHot && hot && sm.hot_on;
+    // upserts always look for frequent keys; mixed batches as above
+    const bool look = kHot && hot && (KIND == KIND_UPSERT || sm.hot_on);
     if (empty && next < end && __popc(parked) < NT) {
       const u64 rank = (u64)__popc(empty & ((1u << lane) - 1u));
       if (ring) {  // the ring's copies (usually complete long ago) become visible to the warp
@@ -2199,8 +2200,9 @@ constexpr u64 kStreamShare = 256;  // ops a streaming warp takes per ticket
 // PATH: how the launch is served, chosen by launch_path: streaming lanes,
 // 32-op chunks, or either, by the table's load (inserts that may lock).  A
 // kernel that holds both spills registers for the one that it does not run
-// (2^22-slot P2HT(M) step: 226 us with both in every kernel, 219 us).
-enum { PATH_EITHER = 0, PATH_STREAM = 1, PATH_CHUNK = 2 };
+// (2^22-slot P2HT(M) step: 226 us with both in every kernel, 219 us).  PATH_SMALL:
+// streaming lanes without HotKeys.
+enum { PATH_EITHER = 0, PATH_STREAM = 1, PATH_CHUNK = 2, PATH_SMALL = 3 };
 template <int SCHEME, bool META, int B, int T, int KIND, bool INS, int PATH>
 __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchArgs a) {
   constexpr bool kHot = (KIND == KIND_UPSERT || KIND == KIND_MIXED) && !INS && PATH == PATH_STREAM;
@@ -2210,12 +2212,10 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
   HotKeys* hot = kHot ? &s_hot : nullptr;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x == 0) s_cnt = 0;
-  // Upserts and one warp of a mixed batch look for frequent keys, in launches of
-  // more than one op per lane (those that take tickets).  Smaller ones last less
-  // than the copies of a hot key take (DoubleHT upserts, us without looking and
-  // with: 300 ops 3.1 and 3.7; Zipf adds, 30,000 ops 9.2 and 10.2, 120,000 27.9 and
-  // 30.0, but 250,000 66 and 47).
-  const bool looks = kHot && a.n > 32ull * kWarps * gridDim.x;
+  // A mixed launch of at most one op per lane does not look for frequent keys
+  // (see launch_path; here by a test, not by a kernel of its own: its warps test
+  // whether to look in any case).
+  const bool looks = kHot && (KIND == KIND_UPSERT || a.n > 32ull * kWarps * gridDim.x);
   if (looks) hot->clear();
   __syncthreads();
   const int op = INS ? (int)OP_INSERT : a.op;
@@ -2298,7 +2298,7 @@ __global__ void __launch_bounds__(kThreads, 4) batch_kernel(TableView tv, BatchA
     const u64 end = a.n - begin < first ? a.n : begin + first;
     s_w[w].base = base;  // the same value on every lane
     s_w[w].share = share;
-    s_w[w].hot_on = looks && (KIND == KIND_UPSERT || w == 0);
+    s_w[w].hot_on = looks && w == 0;
     __syncwarp();
     dcount += warp_stream<SCHEME, META, B, T, KIND>(tv, a, op, lockfree, begin, end, s_w[w], lane, ticket, hot,
                                                     front);
@@ -2362,6 +2362,14 @@ cudaError_t launch_path(const TableView& tv, const BatchArgs& a, cudaStream_t s,
   constexpr int kStream = INS && SCHEME != SCHEME_DOUBLE ? PATH_EITHER : PATH_STREAM;
   const bool rounds = kRounds && (KIND == KIND_QUERY || KIND == KIND_ERASE) && tv.stream != 2;
   const bool locks = kStream == PATH_EITHER && !tv.shortcut;
+  // Upserts of at most one op per lane do not look for frequent keys: they last
+  // less than the copies of a hot key take (DoubleHT, us without looking and with:
+  // 300 ops 3.1 and 3.7; Zipf adds, 30,000 ops 9.2 and 10.2, 120,000 27.9 and 30.0,
+  // but 250,000 66 and 47).  A test in the kernel instead of a second one cost the
+  // large launches 1.4% (8M Zipf adds into a 2^21-slot DoubleHT).
+  if (KIND == KIND_UPSERT && !INS && tv.stream && !rounds && a.n <= 4ull * kThreads * (u64)(num_sms > 0 ? num_sms : 1))
+    return launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, KIND == KIND_UPSERT && !INS ? PATH_SMALL : kStream>>(
+        tv, a, s, num_sms);
   return !tv.stream || rounds || locks
              ? launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, PATH_CHUNK>>(tv, a, s, num_sms)
              : launch_sized<batch_kernel<SCHEME, META, B, T, KIND, INS, kStream>>(tv, a, s, num_sms);
