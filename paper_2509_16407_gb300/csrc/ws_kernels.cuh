@@ -805,8 +805,8 @@ struct TileOps {
   // keys build a 2^16-slot DoubleHT, 5 are in flight per bucket, and the build
   // took 60 us with a new probe after each lost claim, 22 us with this.  (With
   // more lock bits and lane passes, 6.7M inserts into a 2^23-slot IcebergHT(M)
-  // went from 1387 to 650 us.)  Two-choice claims stay where they are (see
-  // claim_limit).  Returns 1 claimed, 2 the slot at idx holds K (plain tables), 0
+  // went from 1387 to 650 us.)  How far a claim may go, see
+  // claim_limit.  Returns 1 claimed, 2 the slot at idx holds K (plain tables), 0
   // lost.
   __device__ static __forceinline__ int lane_claim(const TableView& tv, u64& idx, u64 limit, u64 fk, u64 fv, u64 K,
                                                    u64 V) {
@@ -834,25 +834,30 @@ struct TileOps {
   // chosen one -- `spare` slots emptier than the other when they were read, and
   // one fuller with every lost claim -- is not the fuller one: going on to the
   // end of the bucket left iceberg tables of 2^12 to 2^17 slots with 3 to 13
-  // FULL keys at 0.95, where there were none.  Two choices: not at all.  A key
-  // without a choice that moved on would get in ahead of the keys that have one
-  // and must read both their buckets again after a lost claim: buckets would
-  // fill to the threshold from the keys without a choice, which loses the
-  // evenness that two choices are for wherever several ops are in flight per
-  // bucket.  (The lane passes and restarts of two-choice inserts are limited for
-  // the same reason, see kTwoChoicePasses.)  Keys without a slot when a P2HT is
-  // filled to 0.95 by one insert / one upsert-add call, means of 24 tables (4 of
-  // 2^20), and us per call:
-  //   2^14 slots  moving on to the threshold, 8 passes  18 / 24    106 / 180
-  //               so                                     3 / 3     421 / 385
-  //   2^17 slots  moving on                             52 / 61    174 / 428
-  //               so                                    22 / 23   1412 / 1270
-  //   2^20 slots  moving on                            235 / 295   298 / 877
-  //               so                                   190 / 216   827 / 1698
-  // (one key after another: 2.8, 19 and 138).  From 2^22 slots on the counts are
-  // equal and so takes 1-7% longer (2^22 slots, P2HT(M) 455 -> 514 us).
-  __device__ static __forceinline__ u64 claim_limit(u64 idx, bool choice, u32 spare) {
-    if (SCHEME == SCHEME_P2) return idx + 1;
+  // FULL keys at 0.95, where there were none.  Two choices: while the bucket is
+  // less than half full (8- and 16-slot buckets: not at all).  Nearer to the
+  // threshold a key without a choice that moved on would get in ahead of the keys
+  // that have one and must read both their buckets again after a lost claim:
+  // buckets would fill to the threshold from the keys without a choice, which
+  // loses the evenness that two choices are for wherever several ops are in
+  // flight per bucket.  (The lane passes and restarts of two-choice inserts are
+  // limited for the same reason, see two_choice_passes.)  Keys without a slot when
+  // a P2HT is filled to 0.95 by one insert / one upsert-add call, means of 24
+  // tables (4 of 2^20 and 2^22), and us per call:
+  //   slots   moving on to the threshold    not at all             to half
+  //   2^14     18 / 24     106 / 180       3 / 3   421 / 385     5 / 4    310 / 304
+  //   2^17     52 / 61     174 / 428      22 / 23 1412 / 1270   28 / 36   623 / 602
+  //   2^20    235 / 295    298 / 877     190 / 216 827 / 1698  220 / 205  524 / 1388
+  //   2^22    658 / 765    668 / 1388    662 / 693 713 / 1664  651 / 709  682 / 1646
+  // (one key after another: 2.8, 19, 138 and 549; with a lock bit per bucket 5 / 4,
+  // 32 / 32, 292 / 232 and 700 / 684, in 657 to 5800 us).  A launch that inserts
+  // without the lock (`lone`) leaves the table below 0.6 and may go on to 5/8:
+  // 16,000 keys into an empty 2^16-slot P2HT take 16 us so, 23 us with half.
+  __device__ static __forceinline__ u64 claim_limit(u64 idx, bool choice, u32 spare, bool lone = false) {
+    if (SCHEME == SCHEME_P2) {
+      const u64 to = (idx & ~(u64)(B - 1)) + (u64)(lone ? B / 8 * 5 : B / 2);
+      return B != 32 || idx + 1 > to ? idx + 1 : to;
+    }
     const u64 end = (idx & ~(u64)(B - 1)) + (u64)B;
     return !choice || idx + 1 + spare > end ? end : idx + 1 + spare;
   }
@@ -1218,8 +1223,8 @@ struct TileOps {
       return 1;
     }
     u64 idx = ch == 0 ? ls.ff_idx : ls.f1_idx;
-    if (lane_claim(tv, idx, claim_limit(idx, false, 0), ch == 0 ? ls.ff_k : ls.f1_k, ch == 0 ? ls.ff_v : ls.f1_v, K, V) !=
-        1) {
+    if (lane_claim(tv, idx, claim_limit(idx, false, 0, opk == LW_INSERT_FRONT), ch == 0 ? ls.ff_k : ls.f1_k,
+                   ch == 0 ? ls.ff_v : ls.f1_v, K, V) != 1) {
       fresh = false;
       return -1;
     }
@@ -1359,7 +1364,7 @@ struct TileOps {
         }
       }
     }
-    const int got = lane_claim(tv, fidx, claim_limit(fidx, choice, spare), fk, fv, K, V);
+    const int got = lane_claim(tv, fidx, claim_limit(fidx, choice, spare, opk == LW_INSERT_FRONT), fk, fv, K, V);
     if (got == 0) {
       fresh = false;
       return -1;
@@ -1406,19 +1411,25 @@ constexpr int kWarps = kThreads / 32;
 // tiles take it.  Streaming lanes: restarts of an op for the same reasons.
 constexpr int kChunkPasses = 8;
 constexpr int kLaneRestarts = 4;
-// Two choices.  The tiles serialise the inserts of a bucket's keys, lanes that
-// try again at once favour the keys that read one bucket, so more passes fill a
-// small table less evenly (2^17-slot P2HT to 0.55 and then to 0.95: 37 keys
-// without a slot with 8 passes, 22 with 4; 8-slot buckets, 2^14 slots to 0.9: 292
-// with 8, 237 with 3, 225 with 2, in order 213) but faster (13,107 inserts into a
-// 2^18-slot P2HT at 0.8 load: 205 us with 2, 86 with 4, 78 with 8).  Large tables
-// do not care.  Restarts likewise: upsert-adds that fill a 2^20-slot P2HT to 0.95
-// leave 241 keys with 4 (1059 us), 233 with 3 (1350), 205 with 2 (1867); lanes of
-// metadata tables read a bucket in one wave and lose nothing with 4.
+// Two choices, once an op has seen its first bucket half full: the tiles serialise
+// the inserts of a bucket's keys, lanes that try again at once favour the keys that
+// read one bucket, so more passes fill a small table less evenly (2^17-slot P2HT to
+// 0.55 and then to 0.95: 37 keys without a slot with 8 passes, 22 with 4; 8-slot
+// buckets, whose halves are too few slots to tell, 2^14 slots to 0.9: 292 with 8,
+// 237 with 3, 225 with 2, in order 213) but faster (13,107 inserts into a 2^18-slot
+// P2HT at 0.8 load: 205 us with 2, 86 with 4, 78 with 8).  Restarts likewise:
+// upsert-adds that fill a 2^20-slot P2HT to 0.95 leave 241 keys with 4, 233 with 3,
+// 205 with 2; lanes of metadata tables read a bucket in one wave and lose nothing
+// with 4.  Below half the limits would only cost: 2M Zipf adds into a 2^21-slot P2HT
+// that end at 0.4 load 236 us, 322 with two restarts everywhere.
 template <int B>
-constexpr int kTwoChoicePasses = B == 32 ? 4 : 2;
-template <bool META>
-constexpr int kTwoChoiceRestarts = META ? kLaneRestarts : 2;
+__device__ __forceinline__ int two_choice_passes(u32 occ0) {
+  return B != 32 ? 2 : occ0 < (u32)B / 2 ? kChunkPasses : 4;
+}
+template <int B, bool META>
+__device__ __forceinline__ int two_choice_restarts(u32 occ0) {
+  return META || (B == 32 && occ0 < (u32)B / 2) ? kLaneRestarts : 2;
+}
 
 struct WarpSmem {
   u64 key[32], val[32], out[32], h1[32], h2[32];
@@ -1590,9 +1601,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
   // other than by rounds) never go round again; the loop alone took a quarter
   // more (4M present keys inserted into a 2^26-slot P2HT of 16-slot buckets:
   // 548 us with it, 421 without).
-  constexpr int kPasses = ((KIND == KIND_UPSERT || KIND == KIND_MIXED) && kLaneLock)
-                              ? (SCHEME == SCHEME_P2 ? kTwoChoicePasses<B> : kChunkPasses)
-                              : 1;
+  constexpr int kPasses = ((KIND == KIND_UPSERT || KIND == KIND_MIXED) && kLaneLock) ? kChunkPasses : 1;
   bool again = false;  // run the op through the lane path once more
   if (kRounds) {
     // Whole-bucket rounds: eight buckets per round, one op's bucket per copy
@@ -1718,11 +1727,11 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
                 st = ST_INSERTED;
                 done = true;
               } else {
-                again = true;
+                again = attempt + 1 < two_choice_passes<B>(occ0);
               }
             }
           } else {
-            again = true;  // absent, and this op holds no lock
+            again = attempt + 1 < two_choice_passes<B>(occ0);  // absent, and this op holds no lock
           }
         }
       }
@@ -1815,7 +1824,8 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
           run = false;
           if ((r == -2 && kLaneLock && !locked) ||
               (!fresh && (opk == Ops::LW_INSERT_LOCKED || opk == Ops::LW_INSERT_FREE)))
-            again = true;  // absent without the lock, or a lost claim
+            // absent without the lock, or a lost claim
+            again = SCHEME != SCHEME_P2 || pass + 1 < two_choice_passes<B>(ls.occ0);
           else
             lane_ok = false;
         }
@@ -1895,7 +1905,7 @@ __device__ __forceinline__ int warp_chunk(const TableView& tv, const BatchArgs& 
 // cooperative tiles, which run only when no lane of the warp is active -- so
 // no lane of the warp holds a lock a tile might wait for.  An op that lost a
 // claim, or proved its key absent without the lock, first starts over in its
-// lane (kRestarts).  Refill pauses once enough ops are parked to fill the tiles.
+// lane (kLaneRestarts).  Refill pauses once enough ops are parked to fill the tiles.
 // -------------------------------------------------------------------------
 // Work shares: the warp serves [begin, end), and, unless `ticket` is null,
 // then takes shares of up to sm.share ops (a multiple of 32) of [sm.base, n)
@@ -1911,7 +1921,6 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
   constexpr int NT = 32 / T;
   constexpr unsigned kAll = 0xffffffffu;
   constexpr bool kLaneLock = (SCHEME == SCHEME_DOUBLE) || META || Ops::PRE_SLOTS == B || Ops::kLines;
-  constexpr int kRestarts = SCHEME == SCHEME_P2 ? kTwoChoiceRestarts<META> : kLaneRestarts;
   constexpr bool kHot = KIND == KIND_UPSERT || KIND == KIND_MIXED;
   constexpr u8 kTwice = 0x80;  // in sm.op: the op's key is frequent
   const u64 ks = a.key_stride ? a.key_stride : 1;
@@ -2117,7 +2126,8 @@ __device__ __forceinline__ int warp_stream(const TableView& tv, const BatchArgs&
           if (a.status_out) a.status_out[gi] = st;
           if (st >= ST_FULL) count_failure(tv, st);
           state = L_EMPTY;
-        } else if (((r == -2 && kLaneLock && !locked) || (r == -1 && !fresh)) && restarts < kRestarts) {
+        } else if (((r == -2 && kLaneLock && !locked) || (r == -1 && !fresh)) && 
+                   restarts < (SCHEME == SCHEME_P2 ? two_choice_restarts<B, META>(ls.occ0) : kLaneRestarts)) {
           // Absent without the lock: take it now, or -- its holder may be
           // inserting this very key -- look again without it.  Or a lost
           // claim: the table moved under the snapshot; a held lock stays held.
